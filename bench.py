@@ -566,9 +566,8 @@ def lct_bench(steps: int, peaks=None):
     1024 bins of 32 ps, 2 m wall) against the direct pair sum of Eq. 1 on the
     same surface (one point per pixel at its depth-bin centre, no cosines,
     window from the wall). Reports both times, the shape correlation, and the
-    FFT model's FP64 roofline: two 3-D radix-2 transforms of the
-    (2N) x (2N) x (2M) volume V at 5 V log2(V) flops each, and the 6 V of the
-    spectral product, against the measured FP64 fma rate (2 flops each)."""
+    depth-map model's FP64 roofline: the convolution's N^4 additions against the
+    measured FP64 rate."""
     import torch
     from paper_2506_03747_gb300 import nlos
     n, m, dt, w = 128, 1024, 32e-12, 1.0
@@ -623,18 +622,17 @@ def lct_bench(steps: int, peaks=None):
            "direct_forward_ms": direct_ms, "direct_pairs": n * n * n * n,
            "shape_correlation_lct_vs_direct": corr}
     if peaks and peaks.get("dfma"):
-        vol = (2 * n) * (2 * n) * (2 * m)
-        flops = 2 * 5.0 * vol * math.log2(vol) + 6.0 * vol
+        adds = float(n) ** 4
         props = torch.cuda.get_device_properties(torch.cuda.current_device())
-        peak = props.multi_processor_count * peaks["dfma"] * 2.0 * 2070e6
-        achieved = flops / (lct_ms * 1e-3)
+        peak = props.multi_processor_count * peaks["dfma"] * 2070e6
+        achieved = adds / (lct_ms * 1e-3)
         out["lct_roofline"] = {
-            "bound": "fp64", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
+            "bound": "fp64", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "T add/s",
             "frac": achieved / peak,
-            "peak_basis": f"{props.multi_processor_count} SMs x {peaks['dfma']:.2f} FP64 fma "
-                          f"lanes/clk (measured) x 2 flops x 2070 MHz",
-            "work_basis": "two 3-D radix-2 FFTs of the (2N)^2 (2M) volume, 5 V log2 V flops "
-                          "each, and the spectral product (6 V)"}
+            "peak_basis": f"{props.multi_processor_count} SMs x {peaks['dfma']:.2f} FP64 lanes/clk "
+                          f"(measured) x 2070 MHz",
+            "work_basis": "the convolution over its nonzeros: one FP64 addition a (pixel, scan "
+                          "point) pair"}
     return out
 
 

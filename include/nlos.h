@@ -367,10 +367,13 @@ typedef struct nlos_lct nlos_lct;
 /* Plan of the paper's FFT forward model (the Theory section's 3-D convolution
  * tau = R_t^{-1} F^{-1}[F(R_z V) . F(PSF)], Algorithm 1 steps 1.1-2.2) for an
  * n x n confocal depth map over a wall of half side wall_half_m, with m time
- * bins of bin_width_s (n, m powers of two; n <= 1024, m <= 4096). Computes the
- * PSF (one node per lateral column, slope = w / (m c dt)) and its 3-D FFT on
- * the zero-padded (2n) x (2n) x (2m) grid; holds two complex FP64 volumes of
- * that size on the device (32 n^2 m bytes each). Synchronous. */
+ * bins of bin_width_s (n, m powers of two; n <= 1024, m <= 4096). The PSF has
+ * one node per lateral column (slope = w / (m c dt)) and the volume one voxel
+ * per pixel, so for n^2 <= 900 m the convolution is summed over those nonzeros
+ * (the plan holds the PSF's nodes and the map's voxels, about 24 n^2 bytes);
+ * otherwise the plan holds the PSF's 3-D FFT on the zero-padded
+ * (2n) x (2n) x (2m) grid and a work volume, both complex FP64 on the device
+ * (128 n^2 m bytes each). Synchronous. */
 nlos_status nlos_lct_create(uint32_t n, uint32_t m, double wall_half_m, double bin_width_s,
                             void* cuda_stream, nlos_lct** out);
 

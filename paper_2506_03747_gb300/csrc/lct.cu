@@ -17,10 +17,16 @@
 // by up to M / 1 against M / j^4 at the signal, so FP32 round-off of the
 // transforms (1e-7 of the largest value) would exceed the signal there.
 //
-// Layout: the work volume is [2N][2N][2M] complex (time fastest); each 1-D
-// transform runs in shared memory (bit-reversed load, log2 L radix-2
-// stages); along x and y a CTA takes several lines adjacent in time so that
-// its loads and stores are coalesced.
+// Two forms of the convolution, chosen by the plan's sizes (direct_form):
+//  * direct: both factors are sparse, R_z V with one sample a depth-map pixel
+//    and the PSF with one node a column, so the convolution is N^4 additions
+//    into [N][N][M] (one per pixel and scan point that meet in the window),
+//    with no padding and no transform round-off;
+//  * FFT: for short time axes under wide maps, where N^4 additions cost more
+//    than transforms of the padded volume. Its work volume is [2N][2N][2M]
+//    complex (time fastest); each 1-D transform runs in shared memory
+//    (bit-reversed load, log2 L radix-2 stages); along x and y a CTA takes
+//    several lines adjacent in time so that its loads and stores are coalesced.
 #include "common.cuh"
 
 #include <cmath>
@@ -95,19 +101,26 @@ __global__ void __launch_bounds__(kFftThreads) fft_lines_kernel(const FftArgs a)
   }
 }
 
-// PSF (reading above) written circularly shifted into a zeroed volume.
-__global__ void psf_kernel(double2* vol, LctDims d, double slope4sq) {
-  const uint64_t col = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= (uint64_t)d.n2 * d.n2) return;
-  const uint32_t i = (uint32_t)(col / d.n2), j = (uint32_t)(col % d.n2);
+// PSF (reading above): the z node k of column (i, j); false if it has none.
+__device__ __forceinline__ bool psf_node(const LctDims& d, double slope4sq, uint32_t i, uint32_t j,
+                                         int64_t& k) {
   const double x = -1.0 + 2.0 * i / (double)(d.n2 - 1);
   const double y = -1.0 + 2.0 * j / (double)(d.n2 - 1);
   const double dz = 2.0 / (double)(d.m2 - 1);
   const double target = slope4sq * (x * x + y * y);
   const double kf = rint((target + 1.0) / dz);
-  if (!(kf >= 0.0 && kf < (double)d.m2)) return;
-  const int64_t k = (int64_t)kf;
-  if (fabs(target - (-1.0 + (double)k * dz)) > 0.5 * dz + 1e-12) return;
+  if (!(kf >= 0.0 && kf < (double)d.m2)) return false;
+  k = (int64_t)kf;
+  return !(fabs(target - (-1.0 + (double)k * dz)) > 0.5 * dz + 1e-12);
+}
+
+// The PSF written circularly shifted into a zeroed volume.
+__global__ void psf_kernel(double2* vol, LctDims d, double slope4sq) {
+  const uint64_t col = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= (uint64_t)d.n2 * d.n2) return;
+  const uint32_t i = (uint32_t)(col / d.n2), j = (uint32_t)(col % d.n2);
+  int64_t k;
+  if (!psf_node(d, slope4sq, i, j, k)) return;
   const uint32_t is = (i + d.N) % d.n2;  // origin at node (N, N, M)
   const uint32_t js = (j + d.N) % d.n2;
   const uint32_t ks = (uint32_t)((k + d.M) % d.m2);
@@ -146,6 +159,194 @@ __global__ void time_kernel(const double2* vol, LctDims d, float* tau) {
   tau[e] = (float)(vol[(x * d.n2 + y) * d.m2 + r].x * ((double)d.M / (jd * jd * jd * jd)));
 }
 
+// ---------------------------------------------------------------------------
+// Direct form: tau[x][y][j - 1] = M / j^4 * sum of v(x', y') over the pixels
+// with row(x', y') + k(x - x', y - y') = ceil(j^2 / M) - 1.
+// One warp = a patch of 32 columns (x, y) (lane = column) times one window of
+// time bins, whose FP64 samples it keeps in shared memory as [row][32]. Each
+// lane adds to its own column only, so the additions are plain loads and
+// stores without bank conflicts (red.shared.add.f64 is a compare-and-swap loop
+// here, 45 cycles a warp and SM against 19 of the FP64 pipe). A warp is a CTA
+// of its own, so the hardware balances windows of unequal load. Pixels come
+// in 4 x 4 blocks with the range of their rows; a block that cannot reach the
+// window from the patch is ruled out by one lane.
+// Bound: the FP64 pipe's N^4 additions (1.68 lanes a cycle and SM: 0.53 ms at
+// N = 128), taken about 1.3 times because a pixel's additions from one patch
+// can straddle two windows, and the warps in flight (shared memory holds 12
+// to 24). N = 128, M = 1024: 1.16 ms against 65.7 ms of the FFT form; N = 64:
+// 0.27 against 15.4; N = 16: 0.045 against 0.92. Patches of 32 x 1 columns and
+// 1 x 32 segments of pixels took 1.7 ms. Sums as two FP32 words would take
+// 0.73 ms at the same measured error, but carry 48 bits instead of 53.
+// ---------------------------------------------------------------------------
+constexpr int kDirSide = 4;      // side of a block of pixels
+constexpr int kDirBins = 8;      // windows start at multiples of 8 bins (32-byte stores)
+constexpr int kNoRow = 1 << 28;  // pixel without a surface
+constexpr int kNoNode = 0x7fff;  // PSF column without a node
+
+// Rows of a window. More rows make fewer straddled windows, fewer rows more
+// and smaller warps: 64 against 32 rows take 1.16 / 1.42 ms at N = 128, 0.276 /
+// 0.276 at N = 64, 0.105 / 0.094 at N = 32 and 0.070 / 0.045 at N = 16 (M = 1024).
+int dir_rows(uint32_t N) { return N > 64 ? 64 : 32; }
+
+struct __align__(16) Voxel {
+  double v;
+  int row, pad;
+};
+
+// Bins [j0, j1) (0-based) of a window and the first squared-time row they read.
+struct DirWindow {
+  int j0, j1, row0, rows;
+};
+
+struct DirArgs {
+  const Voxel* vox;        // [N * N]
+  const int2* seg;         // [n_seg] range of the rows of a block of pixels
+  const int16_t* node;     // [2N][2N] time offset of the PSF node, kNoNode: none
+  const double* weight;    // [M] M / j^4
+  const DirWindow* win;
+  float* tau;
+  uint32_t N, M, n_seg, per_row;  // blocks of pixels; per_row along y
+  uint32_t py, px, n_py;   // patch of py columns along y and px along x; patches along y
+};
+
+// Squared-depth sample of 0-based bin z: ceil((z + 1)^2 / M) - 1.
+__host__ __device__ inline int sample_row(int64_t z, int64_t M) {
+  return (int)(((z + 1) * (z + 1) + M - 1) / M - 1);
+}
+
+// R_z V as one (value, row) a pixel, in blocks of side * side pixels, and the
+// row range of each block.
+__global__ void __launch_bounds__(256) voxel_kernel(uint32_t N, uint32_t M, uint32_t side,
+                                                    const int32_t* __restrict__ depth,
+                                                    const float* __restrict__ albedo, Voxel* vox,
+                                                    int2* seg) {
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+  int lo = kNoRow, hi = -1;
+  if (k < N * N) {
+    const uint32_t b = k / (side * side), i = k % (side * side), per_row = N / side;
+    const uint32_t p = (b / per_row * side + i / side) * N + b % per_row * side + i % side;
+    const int32_t z = depth[p];
+    Voxel q{};
+    q.row = kNoRow;
+    if (z >= 0 && z < (int32_t)M) {
+      const double a = albedo ? (double)albedo[p] : 0.5;
+      q.v = a / ((double)(z + 1) * M * M);
+      q.row = lo = hi = sample_row(z, M);
+    }
+    vox[k] = q;
+  }
+  for (uint32_t o = side * side >> 1; o > 0; o >>= 1) {
+    lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (k < N * N && k % (side * side) == 0) seg[k / (side * side)] = make_int2(lo, hi);
+}
+
+// Time offset of the PSF node of each lateral offset (dx, dy) in [-N, N)^2.
+__global__ void node_kernel(int16_t* node, LctDims d, double slope4sq) {
+  const uint32_t col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= d.n2 * d.n2) return;
+  int64_t k;
+  node[col] = psf_node(d, slope4sq, col / d.n2, col % d.n2, k) ? (int16_t)(k - d.M)
+                                                                 : (int16_t)kNoNode;
+}
+
+// The offsets of [a, b] nearest to and farthest from the PSF's centre (which
+// lies between -1 and 0).
+__device__ __forceinline__ int near_offset(int a, int b) { return a > 0 ? a : b < -1 ? b : 0; }
+__device__ __forceinline__ int far_offset(int a, int b) { return -a - 1 > b ? a : b; }
+
+template <int SIDE>
+__global__ void __launch_bounds__(32) direct_kernel(const DirArgs a) {
+  extern __shared__ double hist[];  // [rows of a window][32]
+  const int lane = threadIdx.x;
+  const DirWindow w = a.win[blockIdx.y];
+  const int N = (int)a.N, n2 = 2 * N;
+  const int x0 = (int)(blockIdx.x / a.n_py * a.px), y0 = (int)(blockIdx.x % a.n_py * a.py);
+  const int x1 = min(x0 + (int)a.px, N) - 1, y1 = y0 + (int)a.py - 1;
+  const int xl = x0 + lane / (int)a.py, y = y0 + lane % (int)a.py;
+  const int x = min(xl, x1);  // lanes past the map repeat its last row and store nothing
+  for (int i = 0; i < w.rows; ++i) hist[i * 32 + lane] = 0.0;
+  const int16_t* at = a.node + (x + N) * n2 + y + N;
+  double* h = hist + lane;
+  for (uint32_t s0 = 0; s0 < a.n_seg; s0 += 32) {
+    const uint32_t s = s0 + lane;
+    bool live = false;
+    if (s < a.n_seg) {
+      const int2 r = a.seg[s];
+      const int xs = (int)(s / a.per_row) * SIDE, ys = (int)(s % a.per_row) * SIDE;
+      const int xa = x0 - (xs + SIDE - 1), xb = x1 - xs, ya = y0 - (ys + SIDE - 1), yb = y1 - ys;
+      // the node's offset grows with the distance from the centre; one row of
+      // slack on each side against its rounding
+      const int kn = a.node[(near_offset(xa, xb) + N) * n2 + near_offset(ya, yb) + N];
+      const int kf = a.node[(far_offset(xa, xb) + N) * n2 + far_offset(ya, yb) + N];
+      live = r.x <= r.y && kn != kNoNode && r.x + kn - 1 < w.row0 + w.rows &&
+             r.y + kf + 1 >= w.row0;
+    }
+    for (uint32_t m = __ballot_sync(0xffffffffu, live); m; m &= m - 1) {
+      const uint32_t sl = s0 + __ffs(m) - 1;
+      const int xs = (int)(sl / a.per_row) * SIDE, ys = (int)(sl % a.per_row) * SIDE;
+      const double2* vp = reinterpret_cast<const double2*>(a.vox + sl * (SIDE * SIDE));
+      const int16_t* kp = at - (xs * n2 + ys);
+      double2 q[SIDE * SIDE];
+      int t[SIDE * SIDE];
+#pragma unroll
+      for (int i = 0; i < SIDE * SIDE; ++i) {
+        q[i] = __ldg(vp + i);
+        t[i] = (int)__ldg(kp - (i / SIDE) * n2 - i % SIDE);
+      }
+#pragma unroll
+      for (int i = 0; i < SIDE * SIDE; ++i) {
+        // no node: at least 0x7fff - 4096 rows beyond any window
+        const int r = __double2loint(q[i].y) + t[i] - w.row0;
+        if ((unsigned)r < (unsigned)w.rows) h[r * 32] += q[i].x;
+      }
+    }
+  }
+  // each lane writes 8 bins (32 bytes) of its own column at a time
+  if (xl > x1) return;
+  float* out = a.tau + ((size_t)x * N + y) * a.M;
+  const bool vec = ((reinterpret_cast<uintptr_t>(a.tau) & 15u) == 0) && (a.M % kDirBins) == 0;
+  for (int j = w.j0; j < w.j1; j += kDirBins) {
+    float v[kDirBins];
+#pragma unroll
+    for (int e = 0; e < kDirBins; ++e) {
+      const int je = min(j + e, w.j1 - 1);
+      const int t = (sample_row(je, a.M) - w.row0) * 32;
+      v[e] = (float)(h[t] * a.weight[je]);
+    }
+    if (vec) {
+      reinterpret_cast<float4*>(out + j)[0] = make_float4(v[0], v[1], v[2], v[3]);
+      reinterpret_cast<float4*>(out + j)[1] = make_float4(v[4], v[5], v[6], v[7]);
+    } else {
+      for (int e = 0; e < kDirBins && j + e < w.j1; ++e) out[j + e] = v[e];
+    }
+  }
+}
+
+// Windows of at most max_rows squared-time rows, by bins.
+std::vector<DirWindow> dir_windows(int M, int max_rows) {
+  std::vector<DirWindow> out;
+  for (int j = 0; j < M;) {
+    DirWindow w{j, j, sample_row(j, M), 0};
+    while (w.j1 < M) {
+      const int e = std::min(w.j1 + kDirBins, M);
+      if (sample_row(e - 1, M) - w.row0 + 1 > max_rows) break;
+      w.j1 = e;
+      w.rows = sample_row(e - 1, M) - w.row0 + 1;
+    }
+    out.push_back(w);
+    j = w.j1;
+  }
+  return out;
+}
+
+// The direct form's N^4 additions (4.3 ps each) against the FFT form's passes
+// over 8 N^2 M padded samples (about 490 ps each): direct below N^2 of about
+// 900 M. Measured on both sides of the line: N = 128, M = 64: 1.16 against 3.9
+// ms, M = 16: 1.2 against 1.39; N = 256, M = 64: 18 against 16.
+bool direct_form(uint32_t N, uint32_t M) { return (uint64_t)N * N <= 900ull * M; }
+
 bool pow2(uint32_t v) { return v >= 2 && (v & (v - 1)) == 0; }
 uint32_t ilog2(uint32_t v) {
   uint32_t r = 0;
@@ -163,6 +364,15 @@ struct nlos_lct {
   double2* tw = nullptr;
   uint32_t lmax = 0;
   int device = 0;
+  // direct form
+  bool direct = false;
+  nlos::DirArgs dir{};
+  nlos::Voxel* vox = nullptr;
+  int2* seg = nullptr;
+  int16_t* node = nullptr;
+  double* weight = nullptr;
+  nlos::DirWindow* win = nullptr;
+  uint32_t n_win = 0;
 };
 
 namespace nlos {
@@ -214,6 +424,54 @@ cudaError_t fft3(const nlos_lct& p, double2* vol, int inverse, cudaStream_t st) 
   return cudaSuccess;
 }
 
+void free_plan(nlos_lct* p) {
+  for (void* q : {(void*)p->work, (void*)p->psf_hat, (void*)p->tw, (void*)p->vox, (void*)p->seg,
+                  (void*)p->node, (void*)p->weight, (void*)p->win})
+    if (q) cudaFree(q);
+  delete p;
+}
+
+// The direct form's plan: the PSF's nodes, the time weights and the windows.
+cudaError_t create_direct(nlos_lct* p, double slope4sq, cudaStream_t st) {
+  const LctDims& d = p->d;
+  const uint32_t n_pix = d.N * d.N;
+  DirArgs& a = p->dir;
+  a.N = d.N;
+  a.M = d.M;
+  const uint32_t side = std::min(d.N, (uint32_t)kDirSide);
+  a.n_seg = n_pix / (side * side);
+  a.per_row = d.N / side;
+  a.py = std::min(d.N, 8u);
+  a.px = 32u / a.py;
+  a.n_py = d.N / a.py;
+  const std::vector<DirWindow> win = dir_windows((int)d.M, dir_rows(d.N));
+  std::vector<double> weight(d.M);
+  for (uint32_t z = 0; z < d.M; ++z) {
+    const double j = (double)(z + 1);
+    weight[z] = (double)d.M / (j * j * j * j);
+  }
+  p->n_win = (uint32_t)win.size();
+  cudaError_t e;
+  if ((e = cudaMalloc(&p->vox, sizeof(Voxel) * n_pix)) != cudaSuccess ||
+      (e = cudaMalloc(&p->seg, sizeof(int2) * a.n_seg)) != cudaSuccess ||
+      (e = cudaMalloc(&p->node, sizeof(int16_t) * d.n2 * d.n2)) != cudaSuccess ||
+      (e = cudaMalloc(&p->weight, sizeof(double) * d.M)) != cudaSuccess ||
+      (e = cudaMalloc(&p->win, sizeof(DirWindow) * win.size())) != cudaSuccess ||
+      (e = cudaMemcpyAsync(p->weight, weight.data(), sizeof(double) * d.M, cudaMemcpyHostToDevice,
+                           st)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(p->win, win.data(), sizeof(DirWindow) * win.size(),
+                           cudaMemcpyHostToDevice, st)) != cudaSuccess)
+    return e;
+  a.vox = p->vox;
+  a.seg = p->seg;
+  a.node = p->node;
+  a.weight = p->weight;
+  a.win = p->win;
+  node_kernel<<<(d.n2 * d.n2 + 255) / 256, 256, 0, st>>>(p->node, d, slope4sq);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return cudaStreamSynchronize(st);
+}
+
 }  // namespace
 }  // namespace nlos
 
@@ -237,14 +495,19 @@ nlos_status nlos_lct_create(uint32_t n, uint32_t m, double wall_half_m, double b
   const uint64_t nvol = (uint64_t)p->d.n2 * p->d.n2 * p->d.m2;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   auto fail = [&](cudaError_t e, const char* what) {
-    if (p->work) cudaFree(p->work);
-    if (p->psf_hat) cudaFree(p->psf_hat);
-    if (p->tw) cudaFree(p->tw);
-    delete p;
+    free_plan(p);
     return cuda_error(e, what);
   };
   cudaError_t e = cudaGetDevice(&p->device);
   if (e != cudaSuccess) return fail(e, "cudaGetDevice");
+  const double slope = wall_half_m / ((double)m * kLightSpeed * bin_width_s);
+  p->direct = direct_form(n, m);
+  if (p->direct) {
+    if ((e = create_direct(p, 16.0 * slope * slope, st)) != cudaSuccess)
+      return fail(e, "depth-map model plan");
+    *out = p;
+    return NLOS_OK;
+  }
   if ((e = cudaMalloc(&p->work, sizeof(double2) * nvol)) != cudaSuccess ||
       (e = cudaMalloc(&p->psf_hat, sizeof(double2) * nvol)) != cudaSuccess ||
       (e = cudaMalloc(&p->tw, sizeof(double2) * (p->lmax / 2))) != cudaSuccess)
@@ -259,7 +522,6 @@ nlos_status nlos_lct_create(uint32_t n, uint32_t m, double wall_half_m, double b
                            st)) != cudaSuccess ||
       (e = cudaMemsetAsync(p->psf_hat, 0, sizeof(double2) * nvol, st)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
-  const double slope = wall_half_m / ((double)m * kLightSpeed * bin_width_s);
   const uint64_t cols = (uint64_t)p->d.n2 * p->d.n2;
   psf_kernel<<<(unsigned)((cols + 255) / 256), 256, 0, st>>>(p->psf_hat, p->d, 16.0 * slope * slope);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "psf_kernel");
@@ -276,6 +538,20 @@ nlos_status nlos_lct_forward(nlos_lct* plan, const int32_t* depth_dev, const flo
     return set_error(NLOS_EINVAL, "plan, depth_dev and tau_dev must not be NULL");
   const LctDims& d = plan->d;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  if (plan->direct) {
+    DirArgs a = plan->dir;
+    a.tau = tau_dev;
+    const uint32_t n_pix = d.N * d.N;
+    voxel_kernel<<<(n_pix + 255) / 256, 256, 0, st>>>(
+        d.N, d.M, std::min(d.N, (uint32_t)kDirSide), depth_dev, albedo_dev, plan->vox, plan->seg);
+    NLOS_CUDA_TRY(cudaGetLastError());
+    const size_t smem = sizeof(double) * 32 * dir_rows(d.N);
+    const dim3 grid(a.n_py * ((d.N + a.px - 1) / a.px), plan->n_win);
+    if (d.N >= kDirSide) direct_kernel<kDirSide><<<grid, 32, smem, st>>>(a);
+    else direct_kernel<2><<<grid, 32, smem, st>>>(a);  // a 2 x 2 map
+    NLOS_CUDA_TRY(cudaGetLastError());
+    return NLOS_OK;
+  }
   const uint64_t nvol = (uint64_t)d.n2 * d.n2 * d.m2;
   NLOS_CUDA_TRY(cudaMemsetAsync(plan->work, 0, sizeof(double2) * nvol, st));
   volume_kernel<<<(d.N * d.N + 255) / 256, 256, 0, st>>>(plan->work, d, depth_dev, albedo_dev);
@@ -294,10 +570,7 @@ nlos_status nlos_lct_destroy(nlos_lct* plan) {
   clear_error();
   if (!plan) return set_error(NLOS_EINVAL, "plan is NULL");
   cudaDeviceSynchronize();
-  cudaFree(plan->work);
-  cudaFree(plan->psf_hat);
-  cudaFree(plan->tw);
-  delete plan;
+  free_plan(plan);
   return NLOS_OK;
 }
 
