@@ -11,6 +11,7 @@
 #include "noise_core.cuh"
 #include "reduce_core.cuh"
 
+#include <algorithm>
 #include <cmath>
 
 namespace nlos {
@@ -47,8 +48,10 @@ void jitter_tails(const float* taps, int R, float* tail) {
 }
 
 constexpr int kJitterMaxTaps = 2049;  // R <= 1024 bins
-constexpr int kJitterTile = 1024;
+constexpr int kJitterTile = 1024;     // output bins of a CTA at most (staged form)
+constexpr int kJitterUnrolled = 16;   // radii with a compile-time unrolled form
 
+template <int kTaps>
 struct JitterArgs {
   const float* in;
   float* out;
@@ -56,38 +59,128 @@ struct JitterArgs {
   uint32_t B;
   int R;
   int replicate;  // 1: the edge bins continue outside the trace
-  float taps[kJitterMaxTaps];
+  uint32_t tiles, len;  // runs of a trace and their length (a multiple of a thread's bins)
+  float taps[kTaps];
 };
+using JitterShort = JitterArgs<2 * kJitterUnrolled + 1>;
+using JitterLong = JitterArgs<kJitterMaxTaps>;
 
-// One CTA = one run of kJitterTile output bins of one trace; the input run
-// with its R-bin halo is staged in shared memory (zero outside the trace).
-__global__ void jitter_kernel(const __grid_constant__ JitterArgs a) {
-  extern __shared__ float sm[];  // [kJitterTile + 2R] input
-  const uint32_t tiles_per_trace = (a.B + kJitterTile - 1) / kJitterTile;
-  const uint64_t t = blockIdx.x / tiles_per_trace;
-  const int b0 = (int)(blockIdx.x % tiles_per_trace) * kJitterTile;
+// Two forms, both HBM-bound (8 bytes a bin) once a thread computes several
+// consecutive bins from one window of registers; one bin a thread, each with
+// its own 2R + 1 shared loads, was bound by those loads (16,384 x 1024 bins,
+// R = 7: 86 us; now 22.6 us, 5.9 TB/s).
+//  * rows of 16-byte alignment: each thread takes 8 bins from the 8 + 2R
+//    inputs around them, read straight from global memory (neighbouring
+//    threads' overlap hits L1), so no barrier separates loads and stores;
+//  * other rows (bin counts that are not multiples of 4, unaligned buffers)
+//    and radii above 16: a run of the trace with its halo is staged in shared
+//    memory by coalesced loads, and each thread takes 4 bins from it.
+// Every bin adds its taps in the same order in all forms.
+template <int R>
+__global__ void __launch_bounds__(256) jitter_direct_kernel(const __grid_constant__ JitterShort a) {
+  constexpr int kQ = (R + 3) / 4;  // 16-byte words of halo on each side
+  const uint64_t t = blockIdx.x / a.tiles;
+  const int b0 = (int)(blockIdx.x % a.tiles * a.len + 8 * threadIdx.x);
+  const int B = (int)a.B;
+  if (b0 >= B || 8 * threadIdx.x >= a.len) return;
   const float* row = a.in + t * a.B;
-  for (int i = threadIdx.x; i < kJitterTile + 2 * a.R; i += blockDim.x) {
-    const int b = b0 - a.R + i;
+  float x[8 + 8 * kQ];
+#pragma unroll
+  for (int q = 0; q < 2 + 2 * kQ; ++q) {
+    const int b = b0 + 4 * (q - kQ);  // a multiple of 4: the word lies inside or outside as a whole
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b >= 0 && b < B) {
+      v = __ldg(reinterpret_cast<const float4*>(row + b));
+    } else if (a.replicate) {
+      const float e = __ldg(row + (b < 0 ? 0 : B - 1));
+      v = make_float4(e, e, e, e);
+    }
+    x[4 * q] = v.x;
+    x[4 * q + 1] = v.y;
+    x[4 * q + 2] = v.z;
+    x[4 * q + 3] = v.w;
+  }
+  float acc[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    acc[e] = 0.0f;
+#pragma unroll
+    for (int j = -R; j <= R; ++j) acc[e] = fmaf(a.taps[j + R], x[4 * kQ + e - j], acc[e]);
+  }
+  float4* o = reinterpret_cast<float4*>(a.out + t * a.B + b0);
+  o[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  if (b0 + 4 < B) o[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+}
+
+// RT >= 0: the radius at compile time; -1: a.R.
+template <int RT, class Args>
+__global__ void __launch_bounds__(256) jitter_kernel(const __grid_constant__ Args a) {
+  extern __shared__ __align__(16) float sm[];  // [halo + len + halo], halo a multiple of 4
+  const int R = RT >= 0 ? RT : a.R;
+  const int halo = (R + 3) & ~3;
+  const uint64_t t = blockIdx.x / a.tiles;
+  const int b0 = (int)(blockIdx.x % a.tiles * a.len);
+  const float* row = a.in + t * a.B;
+  for (int i = threadIdx.x; i < (int)a.len + 2 * halo; i += blockDim.x) {
+    const int b = b0 - halo + i;
     if (a.replicate) sm[i] = row[min(max(b, 0), (int)a.B - 1)];
     else sm[i] = (b >= 0 && b < (int)a.B) ? row[b] : 0.0f;
   }
   __syncthreads();
-  float* orow = a.out + t * a.B;
-  for (int i = threadIdx.x; i < kJitterTile; i += blockDim.x) {
-    const int b = b0 + i;
-    if (b >= (int)a.B) break;
-    float acc = 0.0f;
-    // out[b] = sum_j taps[j + R] * in[b - j]; in[b - j] sits at sm[i + R - j]
-    for (int j = -a.R; j <= a.R; ++j) acc = fmaf(a.taps[j + a.R], sm[i + a.R - j], acc);
-    orow[b] = acc;
+  const int o = 4 * (int)threadIdx.x;
+  if (o >= (int)a.len) return;
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  if (RT >= 0) {
+    constexpr int kQ = ((RT >= 0 ? RT : 0) + 3) / 4;
+    float x[4 + 8 * kQ];
+#pragma unroll
+    for (int q = 0; q < 1 + 2 * kQ; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(sm + o + 4 * q);
+      x[4 * q] = v.x;
+      x[4 * q + 1] = v.y;
+      x[4 * q + 2] = v.z;
+      x[4 * q + 3] = v.w;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+      for (int j = -RT; j <= RT; ++j) acc[e] = fmaf(a.taps[j + RT], x[4 * kQ + e - j], acc[e]);
+  } else {
+    // out[b] = sum_j taps[j + R] * in[b - j]; in[b - j] sits at sm[o + e + halo - j]
+    const float* c = sm + o + halo;
+    float x0 = c[R], x1 = c[R + 1], x2 = c[R + 2], x3 = c[R + 3];
+    for (int j = -R; j <= R; ++j) {
+      const float g = a.taps[j + R];
+      acc[0] = fmaf(g, x0, acc[0]);
+      acc[1] = fmaf(g, x1, acc[1]);
+      acc[2] = fmaf(g, x2, acc[2]);
+      acc[3] = fmaf(g, x3, acc[3]);
+      x3 = x2;
+      x2 = x1;
+      x1 = x0;
+      x0 = j < R ? c[-j - 1] : 0.0f;
+    }
+  }
+  float* orow = a.out + t * a.B + b0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (b0 + o + e < (int)a.B) orow[o + e] = acc[e];
+}
+
+template <int R>
+void run_jitter(const JitterShort& a, bool direct, unsigned blocks, unsigned threads, size_t smem,
+                cudaStream_t st) {
+  if constexpr (R >= 0) {
+    if (a.R != R) run_jitter<R - 1>(a, direct, blocks, threads, smem, st);
+    else if (direct) jitter_direct_kernel<R><<<blocks, threads, 0, st>>>(a);
+    else jitter_kernel<R><<<blocks, threads, smem, st>>>(a);
   }
 }
 
 cudaError_t launch_jitter(const float* in, float* out, uint64_t traces, uint32_t B, double sigma,
                           int replicate, cudaStream_t st) {
   if (traces == 0 || B == 0) return cudaSuccess;
-  JitterArgs a;
+  JitterLong a;
   a.in = in;
   a.out = out;
   a.traces = traces;
@@ -96,14 +189,23 @@ cudaError_t launch_jitter(const float* in, float* out, uint64_t traces, uint32_t
   const int k = jitter_taps(sigma, a.taps, kJitterMaxTaps);
   if (k < 0) return cudaErrorInvalidValue;
   a.R = (k - 1) / 2;
-  const uint64_t blocks = traces * ((B + kJitterTile - 1) / kJitterTile);
-  const size_t smem = sizeof(float) * (kJitterTile + 2 * a.R);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(jitter_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+  const bool direct = a.R <= kJitterUnrolled && (B & 3u) == 0 &&
+                      ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
+  // equal runs of a trace, so that no CTA is left with a short remainder
+  const uint32_t per = direct ? 8u : 4u, most = direct ? 256u * 8u : (uint32_t)kJitterTile;
+  a.tiles = (B + most - 1) / most;
+  a.len = ((B + a.tiles - 1) / a.tiles + per - 1) / per * per;
+  a.tiles = (B + a.len - 1) / a.len;
+  const unsigned blocks = (unsigned)(traces * a.tiles);
+  const unsigned threads = (a.len / per + 31u) & ~31u;
+  const size_t smem = direct ? 0 : sizeof(float) * (a.len + 2 * ((a.R + 3) & ~3));
+  if (a.R > kJitterUnrolled) {
+    jitter_kernel<-1><<<blocks, threads, smem, st>>>(a);
+  } else {
+    JitterShort s{in, out, traces, B, a.R, replicate, a.tiles, a.len, {}};
+    std::copy(a.taps, a.taps + k, s.taps);
+    run_jitter<kJitterUnrolled>(s, direct, blocks, threads, smem, st);
   }
-  jitter_kernel<<<(unsigned)blocks, 256, smem, st>>>(a);
   return cudaGetLastError();
 }
 
