@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kAdjTabThreads)
     const float gm = gv * (float)m;
 #pragma unroll
     for (int n = 0; n < kMoments; ++n) {
-      const float d = mt.d[n][m + J];
+      const float d = mt.d[J - m][n];
       h[n] = fmaf(gv, d, h[n]);
       mm[n] = fmaf(gm, d, mm[n]);
     }
@@ -365,7 +365,7 @@ cudaError_t launch_backward(const SceneImpl& sc, const float* grad_tau, float* g
   a.norm = (float)(1.0 / (s * std::sqrt(2.0 * 3.14159265358979323846)));
   a.reach = (float)(6.0 * s);
   a.qstep = (float)std::exp(-1.0 / (s * s));
-  if (use_moments(s)) {
+  if (s >= 2.5 && use_moments(s)) {
     // moment tables: S x (B + 2J) x 48 bytes, stream-ordered, freed after use
     MomTab mt;
     moment_table(s, mt);

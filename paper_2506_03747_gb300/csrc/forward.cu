@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(1024, 1)
   __syncthreads();
   FwdCount cnt;
   uint32_t it = 0;
-  (void)fwd_run_ws<SCAN, COS, MODE, kFwdUnroll, true>(a, 0, 0, sm, (int)a.stages, cnt, &mt, it,
+  (void)fwd_run_ws<SCAN, COS, MODE, MODE == MODE_SPLAT_MOM ? 2 : kFwdUnroll, true>(a, 0, 0, sm, (int)a.stages, cnt, &mt, it,
                                                       a.next_chunk, a.chunk, a.units, 0, &occ);
   if (MODE == MODE_NEAREST_COUNT && cnt.boundary) atomicAdd(a.boundary, cnt.boundary);
   // the count is warp-uniform: one lane adds it, 64 pairs per warp iteration
@@ -66,13 +66,12 @@ __global__ void __launch_bounds__(1024, 1)
 // order of the (tile, window) runs in the list does not matter.
 template <int SCAN, int COS, int MODE>
 __global__ void __launch_bounds__(256) unit_list_kernel(const __grid_constant__ FwdArgs a,
-                                                        int mom_J,
                                                         unsigned long long* __restrict__ list,
                                                         unsigned long long* __restrict__ n_live) {
   __shared__ uint32_t s_warp[8];
   __shared__ unsigned long long s_base;
   const unsigned long long tw = blockIdx.x;
-  const float margin = window_margin<MODE>(a, mom_J);
+  const float margin = window_margin<MODE>(a);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (uint32_t b0 = 0; b0 < a.n_blk; b0 += blockDim.x) {
     const uint32_t blk = b0 + threadIdx.x;
@@ -103,6 +102,46 @@ __global__ void __launch_bounds__(256) unit_list_kernel(const __grid_constant__ 
           unit | ((unsigned long long)dead << kListHalfShift) | ((unsigned long long)rows << 32);
     }
     __syncthreads();
+  }
+}
+
+// Moment form, after the forward: the transients for which the weight kept
+// beyond the splat's cut could exceed 1e-5 of their own peak (far_mass pairs
+// beyond the ends, at most 1.6e-8 of their peak each) are summed again tap by
+// tap. One warp per transient, bound by reading tau once from L2; the sums
+// again are rare (a scan corner whose window holds only tails).
+template <int SCAN, int COS>
+__global__ void __launch_bounds__(256) splat_tail_kernel(const __grid_constant__ FwdArgs a) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t si = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); si < a.S; si += warps) {
+    const ScanPoint sp = a.scan[si];
+    const float far = a.far_mass[sp.row];
+    if (far == 0.f) continue;
+    float* row = a.tau + (size_t)sp.row * a.B;
+    float peak = 0.f;
+    for (uint32_t b = lane; b < a.B; b += 32) peak = fmaxf(peak, row[b]);
+    for (int o = 16; o > 0; o >>= 1) peak = fmaxf(peak, __shfl_xor_sync(0xffffffffu, peak, o));
+    if (!(far * a.norm * 1.6e-8f > 1e-5f * peak)) continue;
+    for (uint32_t b = lane; b < a.B; b += 32) row[b] = 0.f;
+    __syncwarp();
+    for (uint32_t i = lane; i < a.n_pairs; i += 32) {
+      PointPair q;
+      load_pair(a.pairs + i, q);
+      float2 u, w, cn;
+      pair_eval2<SCAN, COS>(q, make_float2(-sp.sx, -sp.sx), make_float2(-sp.sy, -sp.sy),
+                            make_float2(sp.off, sp.off), make_float2(a.kbin, a.kbin), u, w, cn);
+      for (int h = 0; h < 2; ++h) {
+        const float uh = h ? u.y : u.x, wh = h ? w.y : w.x;
+        if (!facing<COS>(h ? cn.y : cn.x) || !(uh > -a.reach && uh < (float)a.B + a.reach)) continue;
+        const int lo = max(0, (int)(floorf(uh - 0.5f - a.reach) + 1.0f));
+        const int hi = min((int)a.B - 1, (int)(ceilf(uh - 0.5f + a.reach) - 1.0f));
+        for (int b = lo; b <= hi; ++b) {
+          const float x = (float)b + 0.5f - uh;
+          red_add_global(row + b, wh * a.norm * expf(-x * x * a.inv2s2));
+        }
+      }
+    }
   }
 }
 
@@ -150,7 +189,19 @@ __global__ void pair_table_kernel(const PairTableArgs t, const ScanPoint* scan, 
 namespace {
 
 using FwdFn = void (*)(FwdArgs, MomTab, OccSet);
-using ListFn = void (*)(FwdArgs, int, unsigned long long*, unsigned long long*);
+using TailFn = void (*)(FwdArgs);
+
+TailFn pick_tail(int scan, int cos) {
+  if (scan == NLOS_CONFOCAL) {
+    if (cos == NLOS_COS_NONE) return splat_tail_kernel<NLOS_CONFOCAL, NLOS_COS_NONE>;
+    if (cos == NLOS_COS_OBJECT) return splat_tail_kernel<NLOS_CONFOCAL, NLOS_COS_OBJECT>;
+    return splat_tail_kernel<NLOS_CONFOCAL, NLOS_COS_OBJECT_WALL>;
+  }
+  if (cos == NLOS_COS_NONE) return splat_tail_kernel<NLOS_NONCONFOCAL, NLOS_COS_NONE>;
+  if (cos == NLOS_COS_OBJECT) return splat_tail_kernel<NLOS_NONCONFOCAL, NLOS_COS_OBJECT>;
+  return splat_tail_kernel<NLOS_NONCONFOCAL, NLOS_COS_OBJECT_WALL>;
+}
+using ListFn = void (*)(FwdArgs, unsigned long long*, unsigned long long*);
 
 template <int SCAN, int COS>
 ListFn pick_list_mode(int mode) {
@@ -198,23 +249,23 @@ FwdFn pick(int scan, int cos, int mode) {
 
 }  // namespace
 
-// D_n[j] = K^(n)(j) / n! for the Gaussian K(x) = exp(-x^2/(2 s^2)) / (s sqrt(2 pi)):
+// D_n[i] = K^(n)(X_i) / (n! q^n) for the Gaussian K(x) = exp(-x^2/(2 s^2)) / (s sqrt(2 pi)):
 // K^(n)(x) = (-1)^n He_n(x/s) K(x) / s^n with the probabilists' Hermite
 // polynomials He_0 = 1, He_1 = t, He_{n+1} = t He_n - n He_{n-1} (FP64).
 void moment_table(double s, MomTab& mt) {
   mt.J = (int)std::ceil(6.0 * s) + 1;
-  for (int j = -mt.J; j <= mt.J; ++j) {
-    const double t = (double)j / s;
+  mt.q = moment_rows_per_bin(s);
+  for (int i = 0; i < (2 * mt.J + 1) * mt.q; ++i) {
+    const double x = 0.5 - (i - mt.J * mt.q + 0.5) / mt.q, t = x / s;
     const double k = std::exp(-0.5 * t * t) / (s * std::sqrt(2.0 * 3.14159265358979323846));
-    double he[kMoments];
+    double he[kMomTerms];
     he[0] = 1.0;
-    if (kMoments > 1) he[1] = t;
-    for (int n = 1; n + 1 < kMoments; ++n) he[n + 1] = t * he[n] - n * he[n - 1];
-    double fact = 1.0, spow = 1.0;
-    for (int n = 0; n < kMoments; ++n) {
-      if (n >= 1) fact *= n;
-      mt.d[n][j + mt.J] = (float)(((n & 1) ? -1.0 : 1.0) * he[n] * k / (spow * fact));
-      spow *= s;
+    he[1] = t;
+    for (int n = 1; n + 1 < kMomTerms; ++n) he[n + 1] = t * he[n] - n * he[n - 1];
+    double scale = 1.0;  // n! (q s)^n
+    for (int n = 0; n < kMomTerms; ++n) {
+      if (n >= 1) scale *= n * mt.q * s;
+      mt.d[i][n] = (float)(((n & 1) ? -1.0 : 1.0) * he[n] * k / scale);
     }
   }
 }
@@ -289,14 +340,11 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
                              8 * 32 + 4 * kRowWords;
   size_t smem;
   if (moments) {
-    // window rows plus 2J halo rows fit the kMomRows moment histograms
-    const uint32_t max_bw = (uint32_t)(kMomRows - 2 * mt.J) & ~3u;
-    a.n_win = (g.B + max_bw - 1) / max_bw;
-    a.bw = ((g.B + a.n_win - 1) / a.n_win + 3) & ~3u;
-    if (a.bw > max_bw) {
-      a.bw = max_bw;
-      a.n_win = (g.B + a.bw - 1) / a.bw;
-    }
+    // windows of at most kMomRows rows over the bins and J beyond each end
+    a.halo = mt.J;
+    const uint32_t max_bw = (uint32_t)(kMomRows / mt.q), bins = g.B + 2u * (uint32_t)a.halo;
+    a.n_win = (bins + max_bw - 1) / max_bw;
+    a.bw = (bins + a.n_win - 1) / a.n_win;
     smem = (size_t)kMoments * kMomRows * kTile * 4 + stage_bytes;
   } else {
     uint32_t max_bw = (uint32_t)(((size_t)optin - stage_bytes) / (kTile * 4)) & ~3u;
@@ -345,12 +393,18 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
     a.list_halves = (NLOS_FWD_LIST_HALVES && a.ppb == 2 * kSubPairs &&
                      a.units < (1ull << kListHalfShift))
                         ? 1u : 0u;
-    e = cudaMallocAsync(reinterpret_cast<void**>(&list), sizeof(unsigned long long) * a.units, st);
+    // the moment form's far_mass lies behind the list
+    const size_t list_bytes = sizeof(unsigned long long) * a.units;
+    e = cudaMallocAsync(reinterpret_cast<void**>(&list),
+                        list_bytes + (moments ? sizeof(float) * g.S : 0), st);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(&sc.scratch->n_live, 0, sizeof(unsigned long long), st);
+    if (moments && e == cudaSuccess) {
+      a.far_mass = reinterpret_cast<float*>(list + a.units);
+      e = cudaMemsetAsync(a.far_mass, 0, sizeof(float) * g.S, st);
+    }
     if (e == cudaSuccess) {
-      lf<<<(unsigned)(a.units / a.n_blk), 256, 0, st>>>(a, moments ? mt.J : 0, list,
-                                                          &sc.scratch->n_live);
+      lf<<<(unsigned)(a.units / a.n_blk), 256, 0, st>>>(a, list, &sc.scratch->n_live);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
@@ -362,10 +416,19 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
     a.list_chunks_per_cta = NLOS_FWD_LIST_CHUNKS_PER_CTA;
     a.list_min_chunk = NLOS_FWD_LIST_MIN;
     a.list_max_chunk = NLOS_FWD_LIST_MAX;
-    a.list_static_pct = NLOS_FWD_LIST_STATIC;
+    // a moment flush costs as much as several units, so its list goes out in
+    // one range per CTA (static 60 / 85 / 100%: 0.72 / 0.69 / 0.66 ms on the
+    // 64 x 64 scan of 65,536 points at sigma = 3.2, 0.17 / 0.19 / 0.13 ms on the 32 x 32
+    // scan of 16,384 points at sigma = 1.6)
+    a.list_static_pct = moments ? NLOS_FWD_MOM_STATIC : NLOS_FWD_LIST_STATIC;
   }
   fn<<<(unsigned)grid, threads, smem, st>>>(a, mt, sc.occ);
   e = cudaGetLastError();
+  if (moments && e == cudaSuccess) {
+    const unsigned blocks = (unsigned)std::min<uint64_t>((g.S + 7) / 8, (uint64_t)sc.num_sms * 8);
+    pick_tail(g.scan_mode, g.cos_mode)<<<blocks, 256, 0, st>>>(a);
+    e = cudaGetLastError();
+  }
   if (list) {
     const cudaError_t ef = cudaFreeAsync(list, st);
     if (e == cudaSuccess) e = ef;

@@ -68,6 +68,9 @@ constexpr int kPairsPerBlock = 256;         // serving kernel: 16 KB per staged 
 #ifndef NLOS_FWD_LIST_MAX
 #define NLOS_FWD_LIST_MAX 32                // ... and at most
 #endif
+#ifndef NLOS_FWD_MOM_STATIC
+#define NLOS_FWD_MOM_STATIC 100             // the same for the moment form, whose flushes cost more
+#endif
 #ifndef NLOS_FWD_CONTIG
 #define NLOS_FWD_CONTIG 1                   // each warp takes a contiguous run of a block's pairs
 #endif
@@ -83,30 +86,53 @@ constexpr int kFwdUnroll = NLOS_FWD_UNROLL;  // (#pragma unroll takes no macro)
 enum { MODE_NEAREST = 0, MODE_NEAREST_COUNT = 1, MODE_SPLAT = 2, MODE_SPLAT_MOM = 3,
        MODE_NEAREST_OCC = 4 /* NEAREST with the occluder visibility test */ };
 
-// Moment form of the splat (standalone forward, sigma >= 2.5 bins): per bin m
-// and scan point, M_n[m] = sum of w c^n over the pairs with floor(u) = m,
-// c = 1/2 - (u - m), n < kMoments; at flush time
-//   tau[b] = sum_n sum_j D_n[j] M_n[b - j],  D_n[j] = K^(n)(j) / n!,
-// the Taylor expansion of the Gaussian K(j + c) about the bin offset j. With
-// 6 moments the truncation error is below 2e-6 of the kernel's peak for sigma
-// >= 2.5 (3e-7 at sigma = 3.2). Each moment histogram has kMomRows rows
-// (window bins plus J on each side).
-constexpr int kMoments = 6;
+// Moment form of the splat (standalone forward and adjoint): the bins are cut
+// into q rows each (q a power of two), and with v = u q, row = floor(v) and
+// c = 1/2 - (v - row), a pair adds w c^n, n < kMoments, to its row's moments;
+// at flush time
+//   tau[b] = sum_n sum_r D_n[r - q b + q J] M_n[r],
+//   D_n[i] = K^(n)(X_i) / (n! q^n),  X_i = 1/2 - (i - q J + 1/2) / q,
+// the Taylor expansion of the Gaussian K about the row's centre. q makes half
+// a row at most 0.16 sigma (0.2 sigma, one row a bin, from sigma = 2.5 up), so
+// that six moments leave a truncation error of at most 3.5e-7 of the kernel's
+// peak (1.3e-6 at sigma = 2.5, 3.1e-7 at 3.2). The shared histogram of each
+// moment has kMomRows rows: a window of kMomRows / q bins, and a flush writes
+// the bins up to J beyond its window. The windows reach J = ceil(6 sigma) + 1
+// bins beyond [0, B), and a bin takes all of the J bins around it, so up to
+// 1.5e-8 of the peak of a pair beyond the splat's cut at |x| = 6 sigma. Where
+// that could show, in a transient that holds little but the cut tails of
+// pairs beyond its ends, splat_tail_kernel sums the taps instead. A pair costs six shared reductions at
+// any sigma, against 12 sigma of its taps: a 32 x 32 scan of 16,384 points at
+// sigma = 1.6 takes 0.139 ms against 2.63 ms pair by pair. Fewer moments on
+// finer rows (five at 0.1 sigma, four at 0.05) reduce less a pair but cut the
+// windows into more: 0.74 and 0.79 ms against 0.68 ms (64 x 64 scan, 65,536
+// points, sigma = 3.2).
+constexpr int kMoments = 6;       // of the forward
+constexpr int kMomTerms = 8;      // terms of the table (the adjoint takes them all)
 constexpr int kMomRows = 256;
 constexpr int kMomMaxJ = 60;
+constexpr int kMomTaps = 144;     // (2J + 1) q at most: 121 at q = 1, 66, 92, 104, 144 at q = 2 .. 16
 constexpr uint32_t kMomStride = kMomRows * 32 * 4;  // bytes between moment histograms
-struct MomTab {
-  int J;                                  // taps j = -J..J
-  float d[kMoments][2 * kMomMaxJ + 1];    // D_n[j + J]
+struct __align__(16) MomTab {
+  int J, q;
+  float d[kMomTaps][kMomTerms];  // D_n[i] as d[i][n]
 };
 
 // Fills mt for the unit-area Gaussian of standard deviation s bins (host).
 void moment_table(double s, MomTab& mt);
 
-// The moment form is used for splat kernels of at least 2.5 bins standard
-// deviation (truncation error <= 1.3e-6 of the peak) whose taps fit MomTab.
+// Rows a bin of the moment form.
+inline int moment_rows_per_bin(double sigma) {
+  int q = 1;
+  if (sigma < 2.5)
+    while (0.5 / q > 0.16 * sigma) q *= 2;
+  return q;
+}
+
+// The moment form is used for splat kernels whose taps fit MomTab (sigma up
+// to 9.8 bins); wider ones run their taps pair by pair.
 inline bool use_moments(double sigma) {
-  return sigma >= 2.5 && (int)std::ceil(6.0 * sigma) + 1 <= kMomMaxJ;
+  return (int)std::ceil(6.0 * sigma) + 1 <= kMomMaxJ;
 }
 
 // Per-thread counters of one forward run, added to the scene scratch at exit.
@@ -139,6 +165,7 @@ struct FwdArgs {
   uint32_t list_static_pct;  // the list's first part (percent) in one contiguous range per CTA
   uint32_t list_halves;      // list entries carry the units' dead halves (ppb = 2 kSubPairs)
   uint32_t n_pairs, S, B, bw, n_win, n_blk, ppb;
+  int halo;          // bins the windows reach beyond [0, B) on each side (moment form: J)
   uint32_t stages;   // staged point blocks (standalone warp-specialised kernel)
   float kbin;        // bins per metre of the scanned leg
   int R;             // jitter radius (NEAREST); 0 = none
@@ -147,6 +174,7 @@ struct FwdArgs {
   float norm;        // splat: 1 / (sigma sqrt(2 pi))
   float reach;       // splat: 6 sigma
   float qstep;       // splat: exp(-1 / sigma^2)
+  float* far_mass;   // moment form: [S] weight of the pairs beyond a transient's ends (zeroed)
   float taps[kMaxTaps];
   int replicate;     // jitter with the edge bins continued outside the window
   float tail[kMaxTaps / 2 + 1];  // replicate corrections (jitter_tails)
@@ -294,6 +322,14 @@ __device__ __forceinline__ bool facing(float cn) {
   return COS == NLOS_COS_NONE ? true : (cn > 0.0f);
 }
 
+// First bin of window `win`, and its bins: the windows tile [-halo, B + halo).
+__device__ __forceinline__ int window_start(const FwdArgs& a, uint32_t win) {
+  return (int)(win * a.bw) - a.halo;
+}
+__device__ __forceinline__ int window_bins(const FwdArgs& a, int w0) {
+  return min((int)a.bw, (int)a.B + a.halo - w0);
+}
+
 // One point's Gaussian splat into this lane's histogram column (bins of the
 // window with |b + 1/2 - u| < 6 sigma), taps by the recurrence
 // K_{b+1} = K_b * rho_b, rho_{b+1} = rho_b * exp(-1/sigma^2), restarted from a
@@ -340,8 +376,8 @@ constexpr unsigned long long kNoUnit = ~0ull;  // end of a run (in FwdSmem::unit
 // warp holds scan point l of the tile.
 struct TileState {
   long long tw = -1;
-  uint32_t w0 = 0;
-  int lim = 0;  // bins of the current window that lie inside [0, B)
+  int w0 = 0;   // first bin of the current window
+  int lim = 0;  // its bins
   float2 sx2, sy2, nsx2, nsy2;
   float2 off2;          // bin offset of the scan point, relative to bin 0
   float2 nw02;          // -(first bin of the window)
@@ -350,20 +386,19 @@ struct TileState {
 };
 
 // Bins beyond the window edges that still matter: 1 for the histogram modes
-// (edge pairs of the boundary count), the splat reach + 1, J + 1 for moments.
+// (edge pairs of the boundary count) and the moment form (whose windows hold
+// the halo themselves), the splat reach + 1 for its taps.
 template <int MODE>
-__device__ __forceinline__ float window_margin(const FwdArgs& a, int mom_J) {
-  return MODE == MODE_SPLAT ? a.reach + 1.0f
-         : MODE == MODE_SPLAT_MOM ? (float)(mom_J + 1)
-                                  : 1.0f;
+__device__ __forceinline__ float window_margin(const FwdArgs& a) {
+  return MODE == MODE_SPLAT ? a.reach + 1.0f : 1.0f;
 }
 
 __device__ __forceinline__ void load_tile(const FwdArgs& a, long long tw, int lane,
                                           TileState& ts, bool confocal, float margin) {
   const uint32_t tile = (uint32_t)(tw / a.n_win);
   ts.tw = tw;
-  ts.w0 = (uint32_t)(tw % a.n_win) * a.bw;
-  ts.lim = (int)min(a.bw, a.B - ts.w0);
+  ts.w0 = window_start(a, (uint32_t)(tw % a.n_win));
+  ts.lim = window_bins(a, ts.w0);
   const uint32_t s = tile * kTile + lane;
   if (s < a.S) {
     const ScanPoint sp = a.scan[s];
@@ -373,7 +408,7 @@ __device__ __forceinline__ void load_tile(const FwdArgs& a, long long tw, int la
     ts.nsy2 = make_float2(-sp.sy, -sp.sy);
     ts.off2 = make_float2(sp.off, sp.off);
     ts.nw02 = make_float2(-(float)ts.w0, -(float)ts.w0);
-    ts.binbase = (uint32_t)kMagicBits + ts.w0;
+    ts.binbase = (uint32_t)(kMagicBits + ts.w0);
     const float o = sp.off - (float)ts.w0;
     // r range of u in [-margin, lim + margin): r = (u - o) / kbin
     const float ik = 1.0f / a.kbin;
@@ -392,7 +427,7 @@ __device__ __forceinline__ void load_tile(const FwdArgs& a, long long tw, int la
     ts.sx2 = ts.sy2 = ts.nsx2 = ts.nsy2 = make_float2(0.f, 0.f);
     ts.off2 = make_float2(-1e30f, -1e30f);  // u -> -inf: never binned
     ts.nw02 = make_float2(0.f, 0.f);
-    ts.binbase = (uint32_t)kMagicBits + ts.w0;
+    ts.binbase = (uint32_t)(kMagicBits + ts.w0);
     ts.r2lo2 = make_float2(1.f, 1.f);      // empty r ranges
     ts.r2hi2 = make_float2(-1.f, -1.f);
   }
@@ -478,8 +513,7 @@ template <int MODE>
 __device__ __forceinline__ void flush_tile(const FwdArgs& a, long long tw, const float* hist,
                                            int warp_rel, int n_warps, int rlo, int rhi) {
   const uint32_t tile = (uint32_t)(tw / a.n_win);
-  const uint32_t win = (uint32_t)(tw % a.n_win);
-  const int w0 = (int)(win * a.bw);
+  const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
   const int R = (MODE == MODE_SPLAT) ? 0 : a.R;
   if (rhi <= rlo) return;
   const int lo = max(0, w0 + rlo - R) & ~3;
@@ -593,7 +627,7 @@ template <int SCAN, int COS, int MODE, int UNROLL>
 __device__ __forceinline__ void compute_block(const FwdArgs& a, const PointPair* blkp, uint32_t n,
                                               int warp_rel, int n_warps, const TileState& ts,
                                               uint32_t col_addr, FwdCount& cnt,
-                                              int mom_J = 0, const OccSet* occ = nullptr,
+                                              int mom_q = 1, const OccSet* occ = nullptr,
                                               uint32_t occ_mask = 0, uint32_t rot = 0) {
   const float2 kbin2 = make_float2(a.kbin, a.kbin);
   const float2 magic2 = make_float2(kMagic, kMagic);
@@ -634,32 +668,22 @@ __device__ __forceinline__ void compute_block(const FwdArgs& a, const PointPair*
 #endif
     float2 u, w;
     pair_finish2<SCAN, COS>(q, r2, cn, ts.off2, kbin2, u, w);
-    // window-relative u for the splat forms (exact: w0 is an integer < 2^24)
-    if (MODE == MODE_SPLAT || MODE == MODE_SPLAT_MOM) u = __fadd2_rn(u, ts.nw02);
     if (MODE == MODE_SPLAT) {
+      // window-relative u (exact: w0 is an integer < 2^24)
+      u = __fadd2_rn(u, ts.nw02);
       if (facing<COS>(cn.x)) splat_one(col_addr, u.x, w.x, ts.lim, a);
       if (facing<COS>(cn.y)) splat_one(col_addr, u.y, w.y, ts.lim, a);
     } else if (MODE == MODE_SPLAT_MOM) {
-      const float2 t = __fadd2_rd(u, magic2);                        // kMagic + floor(u)
-      const float2 fl = __fadd2_rn(t, make_float2(-kMagic, -kMagic));  // floor(u), exact
-      const float2 fr = __fadd2_rn(u, make_float2(-fl.x, -fl.y));      // u - floor(u), exact
+      const float2 v = __fmul2_rn(u, make_float2((float)mom_q, (float)mom_q));  // exact
+      const float2 t = __fadd2_rd(v, magic2);                          // kMagic + floor(v)
+      const float2 fl = __fadd2_rn(t, make_float2(-kMagic, -kMagic));  // floor(v), exact
+      const float2 fr = __fadd2_rn(v, make_float2(-fl.x, -fl.y));      // v - floor(v), exact
       const float2 c = __fadd2_rn(make_float2(0.5f, 0.5f), make_float2(-fr.x, -fr.y));
-      const uint32_t ra = (uint32_t)(__float_as_int(t.x) - kMagicBits + mom_J);
-      const uint32_t rb = (uint32_t)(__float_as_int(t.y) - kMagicBits + mom_J);
-      const uint32_t rows = (uint32_t)(a.bw + 2 * mom_J);
-#if NLOS_FWD_VOTE == 2
-      // one warp-uniform test first: most pairs of a tile fall outside the
-      // window or face away together
-      const bool oka = ra < rows && facing<COS>(cn.x);
-      const bool okb = rb < rows && facing<COS>(cn.y);
-      if (__any_sync(0xffffffffu, oka || okb)) {
-        red_moments<COS>(col_addr + ra * (kTile * 4), w.x, c.x, ra, rows, cn.x);
-        red_moments<COS>(col_addr + rb * (kTile * 4), w.y, c.y, rb, rows, cn.y);
-      }
-#else
+      const uint32_t ra = (uint32_t)(__float_as_int(t.x) - kMagicBits - ts.w0 * mom_q);
+      const uint32_t rb = (uint32_t)(__float_as_int(t.y) - kMagicBits - ts.w0 * mom_q);
+      const uint32_t rows = (uint32_t)(ts.lim * mom_q);
       red_moments<COS>(col_addr + ra * (kTile * 4), w.x, c.x, ra, rows, cn.x);
       red_moments<COS>(col_addr + rb * (kTile * 4), w.y, c.y, rb, rows, cn.y);
-#endif
     } else {
       // kMagic + floor(u), exactly; the window's first bin comes off the
       // integer (floor(u) - w0 = floor(u - w0) for an integer w0)
@@ -724,47 +748,73 @@ __device__ __forceinline__ void compute_block(const FwdArgs& a, const PointPair*
   }
 }
 
-// Moment flush: out[o] = sum_n sum_j D_n[j] M_n[o - w0 - j + J] for the bins o
-// of the window inside [0, B); four bins per thread, one vector reduction.
+// Moment flush: the bins o within J of the window's bins [blo, bhi) that may
+// hold anything, tau[o] += sum_n sum_r D_n[r - q (o - w0) + q J] M_n[r]. A warp
+// takes four consecutive bins at a time (lane = scan point) and, for each row
+// phase, walks the rows k of that phase with the taps of the four bins in
+// registers: bin e meets row k with tap m - e, m = k - o' + J, so each step
+// loads one row and one new tap of each moment for 24 FMAs. (With each bin
+// loading its own rows, four shared loads for the same 24 FMAs, the flushes
+// were the larger part of a splat forward.)
 __device__ __forceinline__ void flush_tile_mom(const FwdArgs& a, const MomTab& mt, long long tw,
-                                               const float* hist, int warp_rel, int n_warps) {
+                                               const float* hist, int warp_rel, int n_warps,
+                                               int blo, int bhi) {
   const uint32_t tile = (uint32_t)(tw / a.n_win);
-  const uint32_t win = (uint32_t)(tw % a.n_win);
-  const int w0 = (int)(win * a.bw);
-  const int lim = (int)min(a.bw, a.B - (uint32_t)w0);
-  const int J = mt.J;
-  const int nq = (lim + 3) >> 2;
+  const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
+  const int J = mt.J, q = mt.q;
+  const int lo = max(0, w0 + blo - J) & ~3;
+  const int hi = bhi > blo ? min((int)a.B, w0 + bhi + J) : lo;
   const int c = threadIdx.x & 31;
   // the transient (output row) of the lane's scan point; none for the padding
   // lanes of a ragged last tile
   const uint32_t si = tile * kTile + c;
   const uint32_t s = si < a.S ? a.scan[si].row : 0xFFFFFFFFu;
-  for (int qi = warp_rel; qi < nq; qi += n_warps) {
-    const int r0 = 4 * qi;  // window-relative output bin
+  for (int o0 = lo + 4 * warp_rel; o0 < hi; o0 += 4 * n_warps) {
+    const int rel = o0 - w0;  // window-relative first bin
     float v[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int k = 0; k < kMoments; ++k) {
-      const float* mk = hist + (size_t)k * kMomRows * kTile;
-      const float* dk = mt.d[k];
+    const int k0 = max(blo, rel - J), k1 = min(bhi, rel + 3 + J + 1);
+    for (int ph = 0; ph < q; ++ph) {
+      float tap[4][kMoments];
+      // taps of bins 1..3 before the first row
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        float acc = v[e];
-        // row of tap j: (r0 + e) - j + J, j = -J..J
-        for (int j = -J; j <= J; ++j) acc = fmaf(dk[j + J], mk[(r0 + e - j + J) * kTile + c], acc);
-        v[e] = acc;
+        const int m = k0 - 1 - rel + J - e;  // becomes bin e + 1's tap at row k0
+#pragma unroll
+        for (int n = 0; n < kMoments; ++n)
+          tap[e][n] = (e < 3 && m >= 0 && m <= 2 * J) ? mt.d[ph + q * m][n] : 0.f;
+      }
+#pragma unroll 4
+      for (int k = k0; k < k1; ++k) {
+        const int m = k - rel + J;
+        const float* h = hist + (size_t)(k * q + ph) * kTile + c;
+#pragma unroll
+        for (int n = 0; n < kMoments; ++n) {
+#pragma unroll
+          for (int e = 3; e > 0; --e) tap[e][n] = tap[e - 1][n];
+          tap[0][n] = m <= 2 * J ? mt.d[ph + q * m][n] : 0.f;
+          const float hn = h[n * kMomRows * kTile];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = fmaf(tap[e][n], hn, v[e]);
+        }
       }
     }
-    const int o0 = w0 + r0;
     if (s < a.S && (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)) {
       float* dst = a.tau + (size_t)s * a.B + o0;
-      if ((a.B & 3u) == 0u && (o0 & 3) == 0) {
+      if ((a.B & 3u) == 0u) {
         red_add_global_v4(dst, make_float4(v[0], v[1], v[2], v[3]));
       } else {
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-          if (r0 + e < lim) red_add_global(dst + e, v[e]);
+          if (o0 + e < (int)a.B) red_add_global(dst + e, v[e]);
       }
     }
   }
+  // the weight of the pairs beyond either end of [0, B) (splat_tail_kernel)
+  float far = 0.f;
+  for (int bin = blo + warp_rel; bin < bhi; bin += n_warps)
+    if (w0 + bin < 0 || w0 + bin >= (int)a.B)
+      for (int ph = 0; ph < q; ++ph) far += hist[(bin * q + ph) * kTile + c];
+  if (s < a.S && far != 0.f) red_add_global(a.far_mass + s, far);
 }
 
 __device__ __forceinline__ void issue_block(const FwdArgs& a, const FwdSmem& sm,
@@ -813,7 +863,7 @@ __device__ __forceinline__ BlockBound block_bound(const FwdArgs& a, uint32_t blk
 // the range of u over the two boxes, window-relative.
 template <int SCAN, int COS>
 __device__ __forceinline__ bool bounds_live(const FwdArgs& a, const TileBound& t,
-                                            const BlockBound& b, uint32_t w0, float lim,
+                                            const BlockBound& b, int w0, float lim,
                                             float margin, float& ulo_out, float& uhi_out) {
   if (b.live == 0.f) return false;
   const float dx = fmaxf(0.f, fmaxf(b.x0 - t.sx1, t.sx0 - b.x1));
@@ -846,8 +896,8 @@ __device__ __forceinline__ bool unit_live(const FwdArgs& a, unsigned long long u
   const unsigned long long tw = unit / a.n_blk;
   const uint32_t blk = (uint32_t)(unit - tw * a.n_blk);
   const uint32_t tile = (uint32_t)(tw / a.n_win);
-  const uint32_t w0 = (uint32_t)(tw % a.n_win) * a.bw;
-  const float lim = (float)min(a.bw, a.B - w0);
+  const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
+  const float lim = (float)window_bins(a, w0);
   const TileBound t = a.tiles[tile];
   const BlockBound b = block_bound(a, blk);
   return bounds_live<SCAN, COS>(a, t, b, w0, lim, margin, ulo_out, uhi_out);
@@ -863,8 +913,8 @@ __device__ __forceinline__ bool unit_live_halves(const FwdArgs& a, unsigned long
   const unsigned long long tw = unit / a.n_blk;
   const uint32_t blk = (uint32_t)(unit - tw * a.n_blk);
   const uint32_t tile = (uint32_t)(tw / a.n_win);
-  const uint32_t w0 = (uint32_t)(tw % a.n_win) * a.bw;
-  const float lim = (float)min(a.bw, a.B - w0);
+  const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
+  const float lim = (float)window_bins(a, w0);
   const TileBound t = a.tiles[tile];
   const uint32_t sb0 = blk * 2u;
   const uint32_t n_sub = (a.n_pairs + kSubPairs - 1) / kSubPairs;
@@ -964,9 +1014,7 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
                            uint32_t& it, unsigned long long* chunk_counter = nullptr,
                            unsigned long long chunk = 0, unsigned long long units_total = 0,
                            uint32_t max_claims = 0, const OccSet* occ = nullptr) {
-  const int mom_J = (MODE == MODE_SPLAT_MOM) ? mt->J : 0;
-  const uint32_t hist_words = (MODE == MODE_SPLAT_MOM) ? (uint32_t)kMoments * kMomRows * kTile
-                                                       : a.bw * kTile;
+  const int mom_q = (MODE == MODE_SPLAT_MOM) ? mt->q : 1;
   __shared__ int s_abort;
   __shared__ uint32_t s_used;  // slots this call used (units + the end mark)
   __shared__ unsigned long long s_list_base;  // first entry of the list's claimed part
@@ -989,15 +1037,13 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
   }
   __syncthreads();
   const bool cull = NLOS_FWD_CULL && a.bounds != nullptr && MODE != MODE_NEAREST_COUNT;
-  // histogram rows tracked per tile (flush and zero only those); the moment
-  // histograms have their own layout and are always handled whole
-  const bool ranged = RANGED && sm.rows != nullptr && cull && MODE != MODE_SPLAT_MOM &&
-                      stages <= kMaxRangedStages;
+  // bins tracked per tile (flush and zero only those)
+  const bool ranged = RANGED && sm.rows != nullptr && cull && stages <= kMaxRangedStages;
   if (warp == 0) {
     // The whole warp walks the units 32 at a time: each lane tests one unit
     // against the bounds (unit_live), then lane 0 stages the live ones in
     // order. Chunk claims (lane 0) run one ahead of their use.
-    const float margin = window_margin<MODE>(a, mom_J);
+    const float margin = window_margin<MODE>(a);
     // list mode: chunks of the live-unit list, sized from its length
     const bool listed = a.unit_list != nullptr && chunk_counter != nullptr &&
                         sm.lane_units != nullptr;
@@ -1173,17 +1219,21 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
         if (tw != ts.tw) {
           named_barrier(1, nthr);  // every consumer is done with the previous tile
           if (ts.tw >= 0) {
-            if (MODE == MODE_SPLAT_MOM) flush_tile_mom(a, *mt, ts.tw, hist, cw, ncw);
+            if constexpr (MODE == MODE_SPLAT_MOM)
+              flush_tile_mom(a, *mt, ts.tw, hist, cw, ncw, (int)(tile_rows & 0xFFFFu),
+                             (int)(tile_rows >> 16));
             else flush_tile<MODE>(a, ts.tw, hist, cw, ncw, (int)(tile_rows & 0xFFFFu),
                                   (int)(tile_rows >> 16));
             named_barrier(1, nthr);
           }
           // zero what the previous tile may have written (everything the first
           // time: the buffer may hold another item's data)
-          const uint32_t z0 = (ranged && ts.tw >= 0) ? (tile_rows & 0xFFFFu) * kTile : 0u;
-          const uint32_t z1 = (ranged && ts.tw >= 0) ? (tile_rows >> 16) * kTile : hist_words;
-          for (uint32_t i = z0 + tid - 32; i < z1; i += nthr) hist[i] = 0.f;
-          load_tile(a, tw, lane, ts, SCAN == NLOS_CONFOCAL, window_margin<MODE>(a, mom_J));
+          const uint32_t per_bin = (uint32_t)(mom_q * kTile);
+          const uint32_t z0 = (ranged && ts.tw >= 0) ? (tile_rows & 0xFFFFu) * per_bin : 0u;
+          const uint32_t z1 = ((ranged && ts.tw >= 0) ? (tile_rows >> 16) : a.bw) * per_bin;
+          for (int n = 0; n < (MODE == MODE_SPLAT_MOM ? kMoments : 1); ++n)
+            for (uint32_t i = z0 + tid - 32; i < z1; i += nthr) hist[n * kMomRows * kTile + i] = 0.f;
+          load_tile(a, tw, lane, ts, SCAN == NLOS_CONFOCAL, window_margin<MODE>(a));
           named_barrier(1, nthr);
         }
         // the producer's running union for this tile, up to this unit
@@ -1196,7 +1246,7 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
         const uint32_t hi = (dead & 2u) ? min(nb, (uint32_t)kSubPairs) : nb;
         compute_block<SCAN, COS, MODE, UNROLL>(a, sm.stage + (size_t)slot * a.ppb + lo,
                                        hi > lo ? hi - lo : 0u, cw, ncw, ts, col_addr, cnt,
-                                       mom_J, occ, (uint32_t)(tag >> kUnitBits), g);
+                                       mom_q, occ, (uint32_t)(tag >> kUnitBits), g);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[slot]);
@@ -1204,7 +1254,9 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
     }
     named_barrier(1, nthr);
     if (ts.tw >= 0) {
-      if (MODE == MODE_SPLAT_MOM) flush_tile_mom(a, *mt, ts.tw, hist, cw, ncw);
+      if constexpr (MODE == MODE_SPLAT_MOM)
+        flush_tile_mom(a, *mt, ts.tw, hist, cw, ncw, (int)(tile_rows & 0xFFFFu),
+                       (int)(tile_rows >> 16));
       else flush_tile<MODE>(a, ts.tw, hist, cw, ncw, (int)(tile_rows & 0xFFFFu),
                             (int)(tile_rows >> 16));
     }
