@@ -137,11 +137,11 @@ typedef struct {
                                  points at a time, pairs that no lane can bin
                                  (outside the window or facing away), after
                                  computing only r^2 and the cosine numerator */
-  uint64_t pairs_tested;      /* pairs of the (scan tile, point block) units
-                                 the forward evaluated at all; the others were
-                                 ruled out from the bounds of the tile's spots
-                                 and of the block's points without touching
-                                 the pairs (counted per unit: 32 x 1024) */
+  uint64_t pairs_tested;      /* pairs of the groups of 16 point pairs that the
+                                 forward evaluated at all; the others were
+                                 ruled out from the bounds of a tile's spots
+                                 and of the group's points without touching
+                                 the pairs (counted per group: 32 x 32) */
 } nlos_stats;
 
 typedef struct nlos_scene nlos_scene;

@@ -79,6 +79,9 @@ struct __align__(16) BlockBound {
   float uo0, uo1, live, pad;
 };
 static_assert(sizeof(BlockBound) == 64, "BlockBound layout");
+// The same record of each group of kGroupPairs packed pairs, of which the
+// forward's producer warp rules out those that the tile cannot bin.
+constexpr uint32_t kGroupPairs = 16;
 
 // Bounds of the scan spots of one tile of kTile scan points (valid ones):
 // spot box and range of the bin offsets off_s.
@@ -188,6 +191,7 @@ struct SceneImpl {
   uint16_t* cell = nullptr;        // [P] Morton cell of each point (ordering scratch)
   uint32_t* cells = nullptr;       // [kOrderCells + 8] counts/cursors + box (ordering scratch)
   BlockBound* bounds = nullptr;    // [ceil(P / 2 / kSubPairs)]
+  BlockBound* groups = nullptr;    // [ceil(P / 2 / kGroupPairs)]
   TileBound* tiles = nullptr;      // [ceil(S / kTile)] of scan_fwd
   OccSet occ{};                    // occluders (host copy; n = 0: none)
   cudaStream_t stream = nullptr;   // creation stream

@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(1024, 1)
   sm.units = reinterpret_cast<unsigned long long*>(sm.bars + 2 * a.stages);
   sm.lane_units = sm.units + a.stages + 1;
   sm.rows = reinterpret_cast<uint32_t*>(sm.lane_units + 32);
+  sm.fill = sm.rows + kRowWords;
   if (threadIdx.x == 0) {
     for (uint32_t i = 0; i < a.stages; ++i) {
       mbar_init(&sm.bars[i], 1);                                 // full
@@ -77,10 +78,9 @@ __global__ void __launch_bounds__(256) unit_list_kernel(const __grid_constant__ 
     const uint32_t blk = b0 + threadIdx.x;
     const unsigned long long unit = tw * a.n_blk + blk;
     float ulo = 0.f, uhi = 0.f;
-    uint32_t dead = 0;
     const bool live =
-        blk < a.n_blk && (a.list_halves
-                              ? unit_live_halves<SCAN, COS>(a, unit, margin, ulo, uhi, dead)
+        blk < a.n_blk && (a.ppb == 2 * kSubPairs
+                              ? unit_live_halves<SCAN, COS>(a, unit, margin, ulo, uhi)
                               : unit_live<SCAN, COS>(a, unit, margin, ulo, uhi));
     const uint32_t rows = live ? unit_rows(ulo, uhi, margin, a.bw) : 0u;
     const uint32_t m = __ballot_sync(0xffffffffu, live);
@@ -98,8 +98,7 @@ __global__ void __launch_bounds__(256) unit_list_kernel(const __grid_constant__ 
     __syncthreads();
     if (live) {
       const uint32_t pos = s_warp[warp] + __popc(m & ((1u << lane) - 1u));
-      list[s_base + pos] =
-          unit | ((unsigned long long)dead << kListHalfShift) | ((unsigned long long)rows << 32);
+      list[s_base + pos] = unit | ((unsigned long long)rows << 32);
     }
     __syncthreads();
   }
@@ -289,6 +288,7 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
   a.pairs_full = &sc.scratch->pairs_full;
   a.pairs_tested = &sc.scratch->pairs_tested;
   a.bounds = sc.bounds;
+  a.groups = sc.groups;
   a.tiles = sc.tiles;
   a.next_chunk = &sc.scratch->next_chunk;
   a.n_pairs = (uint32_t)((g.P + 1) / 2);
@@ -337,7 +337,7 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
   }
   // staged blocks, then full + empty barriers and the unit number of each slot
   const size_t stage_bytes = a.stages * (size_t)a.ppb * sizeof(PointPair) + 24 * a.stages + 64 +
-                             8 * 32 + 4 * kRowWords;
+                             8 * 32 + 4 * kRowWords + 4 * kMaxRangedStages;
   size_t smem;
   if (moments) {
     // windows of at most kMomRows rows over the bins and J beyond each end
@@ -388,11 +388,6 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
   ListFn lf = (NLOS_FWD_CULL && a.bounds) ? pick_list(g.scan_mode, g.cos_mode, mode) : nullptr;
   unsigned long long* list = nullptr;
   if (lf) {
-    // halves (for the list kernel and the forward): two sub-blocks a unit,
-    // and unit numbers that leave bits 30-31 of a list entry free
-    a.list_halves = (NLOS_FWD_LIST_HALVES && a.ppb == 2 * kSubPairs &&
-                     a.units < (1ull << kListHalfShift))
-                        ? 1u : 0u;
     // the moment form's far_mass lies behind the list
     const size_t list_bytes = sizeof(unsigned long long) * a.units;
     e = cudaMallocAsync(reinterpret_cast<void**>(&list),

@@ -62,17 +62,11 @@ constexpr int kPairsPerBlock = 256;         // serving kernel: 16 KB per staged 
 #ifndef NLOS_FWD_LIST_STATIC
 #define NLOS_FWD_LIST_STATIC 75             // live-unit list: percent in static ranges per CTA
 #endif
-#ifndef NLOS_FWD_LIST_HALVES
-#define NLOS_FWD_LIST_HALVES 1              // live-unit list: halves of a unit culled apart
-#endif
 #ifndef NLOS_FWD_LIST_MAX
 #define NLOS_FWD_LIST_MAX 32                // ... and at most
 #endif
 #ifndef NLOS_FWD_MOM_STATIC
 #define NLOS_FWD_MOM_STATIC 100             // the same for the moment form, whose flushes cost more
-#endif
-#ifndef NLOS_FWD_CONTIG
-#define NLOS_FWD_CONTIG 1                   // each warp takes a contiguous run of a block's pairs
 #endif
 #ifndef NLOS_FWD_STAGES
 #define NLOS_FWD_STAGES 3                   // staged blocks in flight (warp-specialised)
@@ -151,6 +145,7 @@ struct FwdArgs {
   unsigned long long* pairs_full;  // pairs past the early out (scene scratch)
   unsigned long long* pairs_tested;  // pairs of staged units (scene scratch)
   const BlockBound* bounds;   // [ceil(n_pairs / kSubPairs)] or null (no unit culling)
+  const BlockBound* groups;   // [ceil(n_pairs / kGroupPairs)], with bounds
   const TileBound* tiles;     // [ceil(S / kTile)]
   unsigned long long* next_chunk;  // standalone launch: chunk counter (zeroed per pass)
   unsigned long long units;   // standalone launch: total units
@@ -163,7 +158,6 @@ struct FwdArgs {
   uint32_t list_chunks_per_cta;  // list chunks per CTA (mean), of the claimed part
   uint32_t list_min_chunk, list_max_chunk;  // list entries per chunk, clamped
   uint32_t list_static_pct;  // the list's first part (percent) in one contiguous range per CTA
-  uint32_t list_halves;      // list entries carry the units' dead halves (ppb = 2 kSubPairs)
   uint32_t n_pairs, S, B, bw, n_win, n_blk, ppb;
   int halo;          // bins the windows reach beyond [0, B) on each side (moment form: J)
   uint32_t stages;   // staged point blocks (standalone warp-specialised kernel)
@@ -362,8 +356,9 @@ struct FwdSmem {
   float* hist;                 // [bw][32]
   PointPair* stage;            // [stages][ppb]
   uint64_t* bars;              // full[stages] then empty[stages] (initialised by the caller)
-  unsigned long long* units;   // [stages]: the unit staged in each slot
+  unsigned long long* units;   // [stages]: the (tile, window) of each slot's pairs
   uint32_t* rows = nullptr;    // [kRowWords] or null: row tracking (see fwd_run_ws)
+  uint32_t* fill = nullptr;    // [stages]: the pairs staged in each slot
   unsigned long long* lane_units = nullptr;  // [32]: the producer lanes' units (list mode)
 };
 // rows: 32 words for the producer's lanes, then one per slot (up to 8 stages)
@@ -540,9 +535,6 @@ __device__ __forceinline__ void flush_tile(const FwdArgs& a, long long tw, const
 #undef NLOS_FLUSH_R
 }
 
-// All pairs of one staged block for this warp (pairs warp_rel, warp_rel +
-// n_warps, ...): evaluate both points of a pair for the lane's scan point and
-// add their weights to the lane's histogram column (or splat them).
 // red.shared.add.f32 [addr + k * kMomStride] of w c^k for the moments k <
 // kMoments of one point, predicated on row < rows and a facing cosine.
 template <int K>
@@ -623,6 +615,9 @@ __device__ __forceinline__ bool occ_seen(const OccSet& o, uint32_t mask, float s
   return true;
 }
 
+// This warp's share of the n pairs of a slot: evaluate both points of a pair for
+// the lane's scan point and add their weights to the lane's histogram column
+// (or splat them).
 template <int SCAN, int COS, int MODE, int UNROLL>
 __device__ __forceinline__ void compute_block(const FwdArgs& a, const PointPair* blkp, uint32_t n,
                                               int warp_rel, int n_warps, const TileState& ts,
@@ -632,24 +627,20 @@ __device__ __forceinline__ void compute_block(const FwdArgs& a, const PointPair*
   const float2 kbin2 = make_float2(a.kbin, a.kbin);
   const float2 magic2 = make_float2(kMagic, kMagic);
   const float2 ikbin_neg = make_float2(-1.0f / a.kbin, -1.0f / a.kbin);
-#if NLOS_FWD_CONTIG
   // a contiguous run of pairs per warp: neighbouring points, so the warps'
   // shared reductions meet different histogram rows at any one time; the
   // short last run rotates over the warps from block to block (rot)
   const uint32_t per = (n + (uint32_t)n_warps - 1u) / (uint32_t)n_warps;
   const uint32_t run = ((uint32_t)warp_rel + rot) % (uint32_t)n_warps;
-  const uint32_t i_begin = min(n, run * per), i_end = min(n, i_begin + per), i_step = 1u;
-#else
-  const uint32_t i_begin = (uint32_t)warp_rel, i_end = n, i_step = (uint32_t)n_warps;
-#endif
+  const uint32_t i_begin = min(n, run * per), i_end = min(n, i_begin + per);
   // iterations of this warp (counted once per block, not per iteration)
-  const uint32_t n_it = i_end > i_begin ? (i_end - 1u - i_begin) / i_step + 1u : 0u;
+  const uint32_t n_it = i_end - i_begin;
   cnt.tested += n_it;
 #if !NLOS_FWD_EARLY
   cnt.full += n_it;
 #endif
 #pragma unroll UNROLL
-  for (uint32_t i = i_begin; i < i_end; i += i_step) {
+  for (uint32_t i = i_begin; i < i_end; ++i) {
     PointPair q;
     load_pair(blkp + i, q);
     float2 r2, cn;
@@ -817,16 +808,6 @@ __device__ __forceinline__ void flush_tile_mom(const FwdArgs& a, const MomTab& m
   if (s < a.S && far != 0.f) red_add_global(a.far_mass + s, far);
 }
 
-__device__ __forceinline__ void issue_block(const FwdArgs& a, const FwdSmem& sm,
-                                            unsigned long long unit, int slot) {
-  const uint32_t blk = (uint32_t)(unit % a.n_blk);
-  const uint32_t first = blk * a.ppb;
-  const uint32_t n = min(a.ppb, a.n_pairs - first);
-  const uint32_t bytes = n * (uint32_t)sizeof(PointPair);
-  mbar_arrive_expect_tx(&sm.bars[slot], bytes);
-  bulk_g2s(sm.stage + (size_t)slot * a.ppb, a.pairs + first, bytes, &sm.bars[slot]);
-}
-
 // max of a * b over a in [a0, a1], b in [b0, b1]
 __device__ __forceinline__ float imax(float a0, float a1, float b0, float b1) {
   return fmaxf(fmaxf(a0 * b0, a0 * b1), fmaxf(a1 * b0, a1 * b1));
@@ -903,13 +884,11 @@ __device__ __forceinline__ bool unit_live(const FwdArgs& a, unsigned long long u
   return bounds_live<SCAN, COS>(a, t, b, w0, lim, margin, ulo_out, uhi_out);
 }
 
-// The same test on each half of a two-sub-block unit: whether the unit is
-// live, its u range over its live halves, and the halves that are not
-// (dead bit h: no pair of half h can reach the window or face a spot).
+// The same test on each sub-block of a unit of two: whether one is live, and
+// the u range over the live ones.
 template <int SCAN, int COS>
 __device__ __forceinline__ bool unit_live_halves(const FwdArgs& a, unsigned long long unit,
-                                                 float margin, float& ulo_out, float& uhi_out,
-                                                 uint32_t& dead) {
+                                                 float margin, float& ulo_out, float& uhi_out) {
   const unsigned long long tw = unit / a.n_blk;
   const uint32_t blk = (uint32_t)(unit - tw * a.n_blk);
   const uint32_t tile = (uint32_t)(tw / a.n_win);
@@ -922,10 +901,30 @@ __device__ __forceinline__ bool unit_live_halves(const FwdArgs& a, unsigned long
   const bool live0 = bounds_live<SCAN, COS>(a, t, a.bounds[sb0], w0, lim, margin, l0, h0);
   const bool live1 = sb0 + 1 < n_sub &&
                      bounds_live<SCAN, COS>(a, t, a.bounds[sb0 + 1], w0, lim, margin, l1, h1);
-  dead = (live0 ? 0u : 1u) | (live1 ? 0u : 2u);
   ulo_out = live0 ? (live1 ? fminf(l0, l1) : l0) : l1;
   uhi_out = live0 ? (live1 ? fmaxf(h0, h1) : h0) : h1;
   return live0 || live1;
+}
+
+// The groups of kGroupPairs pairs of a unit that its tile may bin (bit g: pairs
+// [16 g, 16 g + 16) of the block), one group a lane; the whole warp calls it.
+// cull: whether to test the groups' bounds (else every group of the block).
+template <int SCAN, int COS>
+__device__ __forceinline__ uint32_t unit_groups(const FwdArgs& a, unsigned long long unit,
+                                                float margin, bool cull) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const unsigned long long tw = unit / a.n_blk;
+  const uint32_t blk = (uint32_t)(unit - tw * a.n_blk);
+  const uint32_t first = blk * a.ppb + lane * kGroupPairs;
+  bool live = lane * kGroupPairs < a.ppb && first < a.n_pairs;
+  if (live && cull) {
+    const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
+    float ulo, uhi;
+    live = bounds_live<SCAN, COS>(a, a.tiles[(uint32_t)(tw / a.n_win)],
+                                  a.groups[first / kGroupPairs], w0,
+                                  (float)window_bins(a, w0), margin, ulo, uhi);
+  }
+  return __ballot_sync(0xffffffffu, live);
 }
 
 // Occluders that can meet a segment from a spot of the unit's tile (z = 0)
@@ -978,12 +977,6 @@ __device__ __forceinline__ uint32_t unit_rows(float ulo, float uhi, float margin
 // Units carry the occluder mask of MODE_NEAREST_OCC in their top bits.
 constexpr int kUnitBits = 48;
 constexpr unsigned long long kUnitMask = (1ull << kUnitBits) - 1ull;
-// A staged unit's dead halves (unit_live_halves) in tag bits 46-47, and in
-// bits 30-31 of a live-unit list entry (whose units are then below 2^30).
-constexpr int kHalfShift = 46;
-constexpr unsigned long long kUnitIdMask = (1ull << kHalfShift) - 1ull;
-constexpr int kListHalfShift = 30;
-constexpr uint32_t kListUnitMask = (1u << kListHalfShift) - 1u;
 
 __device__ __forceinline__ void named_barrier(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -994,10 +987,16 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 
 // Warp-specialised run of work units (tile, window, point block) of one job:
-// warp 0 (one lane) stages point blocks with TMA bulk copies into `stages`
-// slots, the other warps evaluate them. The producer writes each slot's unit
-// number beside it (kNoUnit ends the run); the full barrier orders that write
-// before the consumers read it. Units come either from the range [u0, u1)
+// warp 0 stages points with TMA bulk copies into `stages` slots, the other warps
+// evaluate them. The producer tests the bounds of each group of 16 pairs of a
+// unit, one group a lane, and copies the groups that the tile may bin side by
+// side, so a slot holds up to ppb pairs of one (tile, window), of as many units
+// as it takes, and the consumers split them evenly. (Evaluating whole blocks,
+// or halves of them, took 24% more pairs on the 64 x 64 union scene and 35%
+// more on a ragged heightfield; skipping dead groups on the consumers' side
+// left warps waiting for the few that had live ones.) The producer writes each
+// slot's (tile, window) and pair count beside it (kNoUnit ends the run); the
+// full barrier orders them before the consumers read them. Units come either from the range [u0, u1)
 // (chunk_counter == nullptr) or in chunks of `chunk` units claimed from
 // *chunk_counter until units_total is reached (or, with max_claims > 0, after
 // that many claims), so that CTAs that meet cheap units (culled, or most
@@ -1098,8 +1097,23 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
     }
     uint32_t k = 0;
     bool failed = false;
-    long long run_tw = -1;   // lane 0: tile of the last staged unit
-    uint32_t run_rows = 0;   // lane 0: union of the rows of that tile's staged units
+    unsigned long long run_tw = kNoUnit;  // (tile, window) of the last staged unit
+    uint32_t run_rows = 0;   // union of the rows of its units so far
+    unsigned long long slot_tw = kNoUnit; // of the open slot
+    uint32_t fill = 0;       // pairs in the open slot (0: none is open)
+    uint32_t unit_occ = 0, slot_occ = 0;  // occluder masks of the unit and of the open slot
+    // hands the open slot to the consumers
+    auto commit = [&]() {
+      if (lane == 0) {
+        const int slot = (int)((it + k) % (uint32_t)stages);
+        unit_of[slot] = slot_tw | ((unsigned long long)slot_occ << kUnitBits);
+        sm.fill[slot] = fill;
+        if (ranged) s_slot_rows[slot] = run_rows;
+        mbar_arrive(&full[slot]);
+      }
+      ++k;
+      fill = 0;
+    };
     for (;;) {
       if (cur == lim && have_next) {
         cur = min(s_list_base + next * chunk, units_total);
@@ -1129,48 +1143,71 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
         }
       }
       uint32_t mask = __ballot_sync(0xffffffffu, live);
-      if (lane == 0) {
-        while (mask) {
-          const int j = __ffs(mask) - 1;
-          mask &= mask - 1;
+      // the groups of each unit that the tile may bin, packed densely: a slot
+      // takes groups of as many units of one (tile, window) as fill it
+      while (mask && !failed) {
+        const int j = __ffs(mask) - 1;
+        mask &= mask - 1;
+        const unsigned long long unit = listed ? sm.lane_units[j] : cur + j;
+        uint32_t groups = unit_groups<SCAN, COS>(a, unit, margin, cull);
+        if (groups == 0u) continue;
+        const unsigned long long utw = unit / a.n_blk;
+        if (fill > 0 && utw != slot_tw) commit();
+        if (MODE == MODE_NEAREST_OCC) unit_occ = occ_unit_mask(a, unit, *occ);
+        if (ranged) {
+          const uint32_t ur = s_lane_rows[j];
+          if (utw != run_tw) {
+            run_tw = utw;
+            run_rows = ur;
+          } else {
+            run_rows = min(run_rows & 0xFFFFu, ur & 0xFFFFu) |
+                       (max(run_rows >> 16, ur >> 16) << 16);
+          }
+        }
+        const uint32_t first = (uint32_t)(unit - utw * a.n_blk) * a.ppb;  // first pair of the block
+        while (groups) {
           const uint32_t g = it + k;  // slot uses continue across calls
           const int slot = (int)(g % (uint32_t)stages);
-          const uint32_t use = g / (uint32_t)stages;
-          if (use > 0 && !mbar_wait_bounded(&empty[slot], (use - 1) & 1)) {
-            atomicOr(a.err, kErrWaitTimeout);
-            s_abort = 1;
-            failed = true;
-            break;
-          }
-          const unsigned long long raw_unit = listed ? sm.lane_units[j] : cur + j;
-          const unsigned long long unit =
-              (listed && a.list_halves) ? (raw_unit & kListUnitMask) : raw_unit;
-          unsigned long long tag = unit;
-          if (listed && a.list_halves)
-            tag |= (unsigned long long)(raw_unit >> kListHalfShift) << kHalfShift;
-          if (MODE == MODE_NEAREST_OCC)
-            tag |= (unsigned long long)occ_unit_mask(a, unit, *occ) << kUnitBits;
-          if (ranged) {
-            const long long utw = (long long)(unit / a.n_blk);
-            const uint32_t ur = s_lane_rows[j];
-            if (utw != run_tw) {
-              run_tw = utw;
-              run_rows = ur;
-            } else {
-              run_rows = min(run_rows & 0xFFFFu, ur & 0xFFFFu) |
-                         (max(run_rows >> 16, ur >> 16) << 16);
+          if (fill == 0) {  // open the next slot
+            const uint32_t use = g / (uint32_t)stages;
+            if (lane == 0 && use > 0 && !mbar_wait_bounded(&empty[slot], (use - 1) & 1)) {
+              atomicOr(a.err, kErrWaitTimeout);
+              s_abort = 1;
+              failed = true;
             }
-            s_slot_rows[slot] = run_rows;
+            failed = __shfl_sync(0xffffffffu, (int)failed, 0) != 0;
+            if (failed) break;
+            slot_tw = utw;
+            slot_occ = 0;
           }
-          unit_of[slot] = tag;
-          fence_proxy_async_smem();
-          issue_block(a, sm, unit, slot);
-          ++k;
+          slot_occ |= unit_occ;
+          // the lowest groups that fit; only the last group of all is short
+          const uint32_t room = a.ppb / kGroupPairs - fill / kGroupPairs;
+          const uint32_t rank = (uint32_t)__popc(groups & ((1u << lane) - 1u));
+          const bool take = ((groups >> lane) & 1u) && rank < room;
+          const uint32_t taken = __ballot_sync(0xffffffffu, take);
+          const uint32_t top = 31u - (uint32_t)__clz((int)taken);
+          const uint32_t short_by =
+              kGroupPairs - min(kGroupPairs, a.n_pairs - (first + top * kGroupPairs));
+          const uint32_t added = (uint32_t)__popc(taken) * kGroupPairs - short_by;
+          if (lane == 0) mbar_expect_tx(&full[slot], added * (uint32_t)sizeof(PointPair));
+          __syncwarp();
+          if (take) {
+            const uint32_t p0 = first + (uint32_t)lane * kGroupPairs;
+            fence_proxy_async_smem();
+            bulk_g2s(sm.stage + (size_t)slot * a.ppb + fill + rank * kGroupPairs, a.pairs + p0,
+                     min(kGroupPairs, a.n_pairs - p0) * (uint32_t)sizeof(PointPair), &full[slot]);
+          }
+          fill += added;
+          groups &= ~taken;
+          if (fill + kGroupPairs > a.ppb || short_by > 0) commit();
         }
       }
-      if (__shfl_sync(0xffffffffu, (int)failed, 0)) break;
+      if (failed) break;
+      __syncwarp();
       cur += n;
     }
+    if (fill > 0) commit();
     if (lane == 0) {
       if (!failed) {
         // end mark: no copy, a plain arrival completes the slot
@@ -1212,10 +1249,8 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
         break;
       }
       const unsigned long long tag = *(volatile unsigned long long*)&unit_of[slot];
-      const unsigned long long unit = tag == kNoUnit ? kNoUnit : (tag & kUnitIdMask);
-      if (unit != kNoUnit) {
-        const long long tw = (long long)(unit / a.n_blk);
-        const uint32_t blk = (uint32_t)(unit - (unsigned long long)tw * a.n_blk);
+      if (tag != kNoUnit) {
+        const long long tw = (long long)(tag & kUnitMask);
         if (tw != ts.tw) {
           named_barrier(1, nthr);  // every consumer is done with the previous tile
           if (ts.tw >= 0) {
@@ -1238,19 +1273,14 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
         }
         // the producer's running union for this tile, up to this unit
         if (ranged) tile_rows = s_slot_rows[slot];
-        const uint32_t first = blk * a.ppb;
-        const uint32_t nb = min(a.ppb, a.n_pairs - first);
-        // halves of the block the list ruled out are not evaluated
-        const uint32_t dead = (uint32_t)(tag >> kHalfShift) & 3u;
-        const uint32_t lo = (dead & 1u) ? min(nb, (uint32_t)kSubPairs) : 0u;
-        const uint32_t hi = (dead & 2u) ? min(nb, (uint32_t)kSubPairs) : nb;
-        compute_block<SCAN, COS, MODE, UNROLL>(a, sm.stage + (size_t)slot * a.ppb + lo,
-                                       hi > lo ? hi - lo : 0u, cw, ncw, ts, col_addr, cnt,
-                                       mom_q, occ, (uint32_t)(tag >> kUnitBits), g);
+        compute_block<SCAN, COS, MODE, UNROLL>(a, sm.stage + (size_t)slot * a.ppb,
+                                               *(volatile uint32_t*)&sm.fill[slot], cw, ncw, ts,
+                                               col_addr, cnt, mom_q, occ,
+                                               (uint32_t)(tag >> kUnitBits), g);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[slot]);
-      if (unit == kNoUnit) break;
+      if (tag == kNoUnit) break;
     }
     named_barrier(1, nthr);
     if (ts.tw >= 0) {

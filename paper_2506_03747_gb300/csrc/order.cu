@@ -36,9 +36,10 @@ __global__ void __launch_bounds__(256) box_kernel(const float* __restrict__ raw,
 }
 
 __global__ void cell_kernel(const float* __restrict__ raw, uint64_t P, const uint32_t* box,
-                            uint16_t* cell, uint32_t* counts) {
+                            uint16_t* cell, uint32_t* counts, int scan_mode, int cos_mode,
+                            const PackConst pc) {
   cell_range(raw, 0, P, (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
-             (uint64_t)gridDim.x * blockDim.x, box, cell, counts);
+             (uint64_t)gridDim.x * blockDim.x, box, cell, counts, scan_mode, cos_mode, pc);
 }
 
 // The cell counts zeroed and the box words set to their identities (min:
@@ -66,7 +67,7 @@ __global__ void scatter_kernel(const uint16_t* cell, uint64_t P, uint32_t* curso
 __global__ void __launch_bounds__(kSubPairs) pack_bounds_kernel(
     const float* __restrict__ raw, uint64_t P, int scan_mode, int cos_mode, const PackConst pc,
     const uint32_t* __restrict__ perm, PointPair* pairs, unsigned int* err,
-    BlockBound* bounds, const __grid_constant__ OccSet occ) {
+    BlockBound* bounds, BlockBound* groups, const __grid_constant__ OccSet occ) {
   static_assert(kSubPairs % 32 == 0 && kSubPairs <= 1024, "one thread per pair of a sub-block");
   __shared__ float red[kSubPairs / 32][15];
   const uint64_t n_pairs = (P + 1) / 2;
@@ -98,8 +99,12 @@ __global__ void __launch_bounds__(kSubPairs) pack_bounds_kernel(
       if (kq != 0.f || na != 0.f || nb != 0.f || nc != 0.f) live = 1.f;
     }
   }
-  bound_warp_reduce(lo, hi, live);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // half a warp is one group
+  static_assert(kGroupPairs == 16, "one group per half warp");
+  bound_warp_reduce<16>(lo, hi, live);
+  if ((lane & 15) == 0 && k < n_pairs) groups[k / kGroupPairs] = bound_record(lo, hi, live);
+  bound_combine(lo, hi, live, 16);
   if (lane == 0) {
     for (int c = 0; c < 7; ++c) {
       red[warp][c] = lo[c];
@@ -133,18 +138,19 @@ cudaError_t launch_order_pack(SceneImpl& s, cudaStream_t st) {
   const uint64_t P = g.P;
   if (P == 0) return cudaSuccess;
   uint32_t* counts = s.cells;
+  const PackConst pc = pack_const(s.params.laser_x, s.params.laser_y, 1.0 / g.cdt);
   uint32_t* box = s.cells + kOrderCells;
   order_init_kernel<<<32, 256, 0, st>>>(counts, box);
   box_kernel<<<grid_for(P, 2048, s.num_sms), 256, 0, st>>>(s.raw_points, P, box);
-  cell_kernel<<<grid_for(P, 256, s.num_sms), 256, 0, st>>>(s.raw_points, P, box, s.cell, counts);
+  cell_kernel<<<grid_for(P, 256, s.num_sms), 256, 0, st>>>(s.raw_points, P, box, s.cell, counts,
+                                                              g.scan_mode, g.cos_mode, pc);
   scan_kernel<<<1, 1024, 0, st>>>(counts);
   scatter_kernel<<<grid_for(P, 256, s.num_sms), 256, 0, st>>>(s.cell, P, counts, s.perm);
   const uint64_t n_pairs = (P + 1) / 2;
-  const PackConst pc = pack_const(s.params.laser_x, s.params.laser_y, 1.0 / g.cdt);
   const uint64_t n_sub = (n_pairs + kSubPairs - 1) / kSubPairs;
   pack_bounds_kernel<<<(unsigned)n_sub, kSubPairs, 0, st>>>(
       s.raw_points, P, g.scan_mode, g.cos_mode, pc, s.perm, s.pairs, &s.scratch->err,
-      s.bounds, s.occ);
+      s.bounds, s.groups, s.occ);
   return cudaGetLastError();
 }
 

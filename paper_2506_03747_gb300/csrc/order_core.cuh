@@ -10,6 +10,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "pack_core.cuh"
 
 namespace nlos {
 
@@ -92,9 +93,28 @@ __device__ __forceinline__ void box_range(const float* __restrict__ raw, uint64_
   __syncthreads();
 }
 
+// Can a point carry weight? False only where its packed weight factor is zero:
+// albedo or area 0, or (non-confocal scans with object cosines) facing away
+// from the laser spot, by the arithmetic of pack_pair_value.
+__device__ __forceinline__ bool point_live(const float4& r0, const float4& r1, int scan_mode,
+                                           int cos_mode, const PackConst& pc) {
+  bool live = r1.z * r1.w != 0.f;
+  if (scan_mode == NLOS_NONCONFOCAL && cos_mode != NLOS_COS_NONE) {
+    const LaserLeg g = laser_leg(r0.x, r0.y, r0.z, pc);
+    live = live && -fmaf(r0.w, g.vx, fmaf(r1.x, g.vy, r1.y * r0.z)) > 0.f;
+  }
+  return live;
+}
+
+// Points that carry no weight go to the last cells (kDeadCells of them, so
+// that their counters are not one address), so that whole blocks of them are
+// ruled out by their bounds.
+constexpr uint32_t kDeadCells = 64;
+
 __device__ __forceinline__ void cell_range(const float* __restrict__ raw, uint64_t b, uint64_t e,
                                            uint64_t t0, uint64_t stride, const uint32_t* box,
-                                           uint16_t* cell, uint32_t* counts) {
+                                           uint16_t* cell, uint32_t* counts, int scan_mode,
+                                           int cos_mode, const PackConst& pc) {
   float lo[3], hi[3], inv[3];
   for (int c = 0; c < 3; ++c) {
     lo[c] = ord_float(box[c]);
@@ -102,7 +122,12 @@ __device__ __forceinline__ void cell_range(const float* __restrict__ raw, uint64
   }
   box_scale(lo, hi, inv);
   for (uint64_t i = b + t0; i < e; i += stride) {
-    const uint32_t k = cell_of(raw[8 * i], raw[8 * i + 1], raw[8 * i + 2], lo, inv);
+    float r[8];
+    load_point(raw + 8 * i, r);
+    const float4 r0 = make_float4(r[0], r[1], r[2], r[3]), r1 = make_float4(r[4], r[5], r[6], r[7]);
+    const uint32_t k = point_live(r0, r1, scan_mode, cos_mode, pc)
+                           ? cell_of(r0.x, r0.y, r0.z, lo, inv)
+                           : kOrderCells - kDeadCells + (uint32_t)(i / 32 % kDeadCells);
     cell[i] = (uint16_t)k;
     // one atomic per distinct cell of the warp: points given in grid or scan
     // order put a warp's 32 points in one or two cells, whose counter the

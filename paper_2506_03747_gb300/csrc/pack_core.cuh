@@ -204,14 +204,19 @@ __device__ __forceinline__ void bound_point(const float* r, int scan_mode, int c
   if (w) live = 1.f;
 }
 
-__device__ __forceinline__ void bound_warp_reduce(float lo[7], float hi[7], float& live) {
-  for (int o = 16; o > 0; o >>= 1) {
-    for (int c = 0; c < 7; ++c) {
-      lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-      hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-    }
-    live = fmaxf(live, __shfl_xor_sync(0xffffffffu, live, o));
+// One step of a butterfly reduction of bounds, at lane distance o.
+__device__ __forceinline__ void bound_combine(float lo[7], float hi[7], float& live, int o) {
+  for (int c = 0; c < 7; ++c) {
+    lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
+    hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
   }
+  live = fmaxf(live, __shfl_xor_sync(0xffffffffu, live, o));
+}
+
+// Bounds over each WIDTH consecutive lanes.
+template <int WIDTH = 32>
+__device__ __forceinline__ void bound_warp_reduce(float lo[7], float hi[7], float& live) {
+  for (int o = WIDTH / 2; o > 0; o >>= 1) bound_combine(lo, hi, live, o);
 }
 
 __device__ __forceinline__ BlockBound bound_record(const float lo[7], const float hi[7],
@@ -224,12 +229,13 @@ __device__ __forceinline__ BlockBound bound_record(const float lo[7], const floa
 }
 
 // Bounds of sub-block sb (points 2 kSubPairs sb .. in packed order) by one
-// warp; lane 0 writes *out. Same per-point quantities as pack_pair.
+// warp, and of its groups (one a step of 32 points); lane 0 writes out[sb] and
+// the groups' records. Same per-point quantities as pack_pair.
 __device__ __forceinline__ void block_bound_warp(const float* __restrict__ raw, uint64_t P,
                                                  uint64_t sb, int scan_mode, int cos_mode,
                                                  const PackConst& pc,
                                                  const uint32_t* __restrict__ perm,
-                                                 BlockBound* out) {
+                                                 BlockBound* out, BlockBound* groups) {
   const int lane = threadIdx.x & 31;
   float lo[7], hi[7];
   for (int c = 0; c < 7; ++c) {
@@ -237,12 +243,27 @@ __device__ __forceinline__ void block_bound_warp(const float* __restrict__ raw, 
     hi[c] = -3.0e38f;
   }
   float live = 0.f;
+  static_assert(kGroupPairs == 16, "a group is one step of the warp");
   const uint64_t first = sb * 2 * kSubPairs;
   const uint64_t last = min(P, first + 2 * kSubPairs);
-  for (uint64_t i = first + lane; i < last; i += 32)
-    bound_point(raw + 8 * (perm ? (uint64_t)perm[i] : i), scan_mode, cos_mode, pc, lo, hi, live);
-  bound_warp_reduce(lo, hi, live);
-  if (lane == 0) *out = bound_record(lo, hi, live);
+  for (uint64_t g0 = first; g0 < last; g0 += 2 * kGroupPairs) {
+    float gl[7], gh[7], gv = 0.f;
+    for (int c = 0; c < 7; ++c) {
+      gl[c] = 3.0e38f;
+      gh[c] = -3.0e38f;
+    }
+    const uint64_t i = g0 + lane;
+    if (i < last)
+      bound_point(raw + 8 * (perm ? (uint64_t)perm[i] : i), scan_mode, cos_mode, pc, gl, gh, gv);
+    bound_warp_reduce(gl, gh, gv);
+    if (lane == 0) groups[g0 / (2 * kGroupPairs)] = bound_record(gl, gh, gv);
+    for (int c = 0; c < 7; ++c) {
+      lo[c] = fminf(lo[c], gl[c]);
+      hi[c] = fmaxf(hi[c], gh[c]);
+    }
+    live = fmaxf(live, gv);
+  }
+  if (lane == 0) out[sb] = bound_record(lo, hi, live);
 }
 
 }  // namespace nlos

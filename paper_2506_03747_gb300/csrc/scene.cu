@@ -161,7 +161,8 @@ nlos_status scene_create_rows(const nlos_params* params, const float* pts, uint6
   auto fail = [&](nlos_status code, const std::string& msg) {
     for (void* q : {(void*)s.pairs, (void*)s.scan, (void*)s.scan_fwd, (void*)s.scratch,
                     (void*)s.raw_points,
-                    (void*)s.perm, (void*)s.cell, (void*)s.cells, (void*)s.bounds, (void*)s.tiles})
+                    (void*)s.perm, (void*)s.cell, (void*)s.cells, (void*)s.bounds, (void*)s.groups,
+                    (void*)s.tiles})
       if (q) cudaFree(q);
     delete sc;
     return set_error(code, msg);
@@ -186,7 +187,10 @@ nlos_status scene_create_rows(const nlos_params* params, const float* pts, uint6
       (P > 0 && (e = cudaMalloc(&s.perm, sizeof(uint32_t) * P)) != cudaSuccess) ||
       (P > 0 && (e = cudaMalloc(&s.cell, sizeof(uint16_t) * P)) != cudaSuccess) ||
       (P > 0 && (e = cudaMalloc(&s.cells, sizeof(uint32_t) * (kOrderCells + 8))) != cudaSuccess) ||
-      (P > 0 && (e = cudaMalloc(&s.bounds, sizeof(BlockBound) * n_sub)) != cudaSuccess))
+      (P > 0 && (e = cudaMalloc(&s.bounds, sizeof(BlockBound) * n_sub)) != cudaSuccess) ||
+      (P > 0 && (e = cudaMalloc(&s.groups, sizeof(BlockBound) *
+                                               ((n_pairs + kGroupPairs - 1) / kGroupPairs))) !=
+                    cudaSuccess))
     return fail(NLOS_ENOMEM, std::string("device allocation failed: ") + cudaGetErrorString(e));
 
   e = cudaMemsetAsync(s.scratch, 0, sizeof(SceneScratch), st);
@@ -302,7 +306,8 @@ nlos_status scene_destroy(nlos_scene* sc) {
   if (s.scratch && (e2 = cudaFree(s.scratch)) != cudaSuccess) e = e2;
   if (s.raw_points && (e2 = cudaFree(s.raw_points)) != cudaSuccess) e = e2;
   if (s.base_points && (e2 = cudaFree(s.base_points)) != cudaSuccess) e = e2;
-  for (void* q : {(void*)s.perm, (void*)s.cell, (void*)s.cells, (void*)s.bounds, (void*)s.tiles})
+  for (void* q : {(void*)s.perm, (void*)s.cell, (void*)s.cells, (void*)s.bounds, (void*)s.groups,
+                    (void*)s.tiles})
     if (q && (e2 = cudaFree(q)) != cudaSuccess) e = e2;
   delete sc;
   if (e != cudaSuccess) return cuda_error(e, "cudaFree");

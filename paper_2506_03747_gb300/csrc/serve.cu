@@ -289,7 +289,7 @@ __device__ __noinline__ void pack_item(const JobDesc& j, uint64_t b, uint64_t e)
   const uint64_t sb_end = (e + kSubPairs - 1) / kSubPairs;
   for (uint64_t sb = b / kSubPairs + (threadIdx.x >> 5); sb < sb_end; sb += blockDim.x >> 5)
     block_bound_warp(j.raw, j.P, sb, j.scan_mode, j.cos_mode, j.pc, j.perm,
-                     const_cast<BlockBound*>(j.fwd.bounds) + sb);
+                     const_cast<BlockBound*>(j.fwd.bounds), const_cast<BlockBound*>(j.fwd.groups));
 }
 
 // full[i] (one arrival: the producer's expect_tx) and empty[i] (one arrival
@@ -309,7 +309,9 @@ __global__ void __launch_bounds__(kServeThreads, 1) serve_kernel(const ServeArgs
   sm.stage = reinterpret_cast<PointPair*>(smem + (size_t)kCapBw * kTile * 4);
   sm.bars = reinterpret_cast<uint64_t*>(sm.stage + kServeStages * kServePpb);
   sm.units = reinterpret_cast<unsigned long long*>(sm.bars + 2 * kServeStages);
-  JobDesc* jd = reinterpret_cast<JobDesc*>(sm.units + kServeStages + 1);
+  sm.fill = reinterpret_cast<uint32_t*>(sm.units + kServeStages + 1);
+  JobDesc* jd = reinterpret_cast<JobDesc*>(sm.fill + 4);
+  static_assert(kServeStages <= 4, "one fill word a stage");
   __shared__ WorkItem s_item;
   __shared__ unsigned long long s_idx;
   __shared__ int s_lane;  // ring of the claimed item
@@ -452,7 +454,7 @@ __global__ void __launch_bounds__(kServeThreads, 1) serve_kernel(const ServeArgs
         break;
       case K_CELL:
         cell_range(jd->raw, item.begin, item.end, tid, blockDim.x, jd->cells + kOrderCells,
-                   jd->cell, jd->cells);
+                   jd->cell, jd->cells, jd->scan_mode, jd->cos_mode, jd->pc);
         break;
       case K_SCAN:
         scan_cells(jd->cells, reinterpret_cast<uint32_t*>(sm.hist));
@@ -530,6 +532,7 @@ struct Request {
   uint32_t* counts = nullptr;
   SceneScratch* scratch = nullptr;
   BlockBound* bounds = nullptr;
+  BlockBound* groups = nullptr;
   TileBound* tiles = nullptr;
   SceneScratch* h_scratch = nullptr;  // pinned copy at completion (the slot's pool entry)
   cudaEvent_t ev = nullptr;
@@ -611,6 +614,8 @@ void carve(Request* r) {
   size_t o_scr = take(sizeof(SceneScratch));
   const uint64_t n_sub = (n_pairs + kSubPairs - 1) / kSubPairs;
   size_t o_bnd = take(sizeof(BlockBound) * (n_sub ? n_sub : 1));
+  const uint64_t n_grp = (n_pairs + kGroupPairs - 1) / kGroupPairs;
+  size_t o_grp = take(sizeof(BlockBound) * (n_grp ? n_grp : 1));
   size_t o_til = take(sizeof(TileBound) * ((g.S + kTile - 1) / kTile));
   r->bytes = off;
   if (!r->dev) return;
@@ -624,6 +629,7 @@ void carve(Request* r) {
   r->counts = g.noise_mode != NLOS_NOISE_NONE ? reinterpret_cast<uint32_t*>(r->dev + o_cnt) : nullptr;
   r->scratch = reinterpret_cast<SceneScratch*>(r->dev + o_scr);
   r->bounds = reinterpret_cast<BlockBound*>(r->dev + o_bnd);
+  r->groups = reinterpret_cast<BlockBound*>(r->dev + o_grp);
   r->tiles = reinterpret_cast<TileBound*>(r->dev + o_til);
 }
 
@@ -640,6 +646,7 @@ void fill_job(Server& sv, Request* r, JobDesc& j) {
   a.pairs_full = &r->scratch->pairs_full;
   a.pairs_tested = &r->scratch->pairs_tested;
   a.bounds = r->bounds;
+  a.groups = r->groups;
   a.tiles = r->tiles;
   a.n_pairs = (uint32_t)((g.P + 1) / 2);
   a.S = (uint32_t)g.S;
