@@ -214,15 +214,14 @@ nlos_status nlos_detect(nlos_scene* scene, const float* tau_dev, uint32_t* count
     return set_error(NLOS_EINVAL, "counts_dev given but noise_mode is NONE");
   cudaStream_t st = as_stream(cuda_stream);
   // reset the reduction results (not the forward's counters)
-  NLOS_CUDA_TRY(cudaMemsetAsync(&s.scratch->peak_bits, 0, sizeof(unsigned int), st));
-  NLOS_CUDA_TRY(cudaMemsetAsync(&s.scratch->sum, 0,
-                                offsetof(SceneScratch, pairs_full) - offsetof(SceneScratch, sum), st));
+  NLOS_CUDA_TRY(cudaMemsetAsync(&s.scratch->peak_bits, 0,
+                                sizeof(SceneScratch) - kScratchDetectOffset, st));
   NLOS_CUDA_TRY(launch_reduce(tau_dev, g.S, g.B, energy_dev, s.scratch, st));
   if (counts_dev)
     NLOS_CUDA_TRY(launch_noise_scene(tau_dev, g.S * (uint64_t)g.B, s.scratch, g.noise_mode,
                                      s.params.peak_photons, s.params.dark_per_bin,
                                      s.params.nr_db, s.params.seed, s.params.stream_tag,
-                                     counts_dev, st, first_bin(g)));
+                                     counts_dev, st, first_bin(g), nullptr, 0, s.noise_lists));
   return NLOS_OK;
 }
 
@@ -238,11 +237,13 @@ nlos_status nlos_noise_part(nlos_scene* scene, const float* tau_dev, uint32_t* c
   if (g.noise_mode == NLOS_NOISE_NONE) return set_error(NLOS_EINVAL, "noise_mode is NONE");
   if (cube_bins < g.S * (uint64_t)g.B)
     return set_error(NLOS_EINVAL, "cube_bins is smaller than the scene's own bins");
+  NLOS_CUDA_TRY(cudaMemsetAsync(s.scratch->deferred, 0, sizeof(s.scratch->deferred),
+                                as_stream(cuda_stream)));
   NLOS_CUDA_TRY(launch_noise_scene(tau_dev, g.S * (uint64_t)g.B, s.scratch, g.noise_mode,
                                    s.params.peak_photons, s.params.dark_per_bin, s.params.nr_db,
                                    s.params.seed, s.params.stream_tag, counts_dev,
                                    as_stream(cuda_stream), first_bin(g), cube_stats_dev,
-                                   cube_bins));
+                                   cube_bins, s.noise_lists));
   return NLOS_OK;
 }
 

@@ -94,27 +94,31 @@ static_assert(sizeof(TileBound) == 32, "TileBound layout");
 // of the scene's bounding box, so that a packed block holds nearby points
 // and its bounds are tight.
 constexpr uint32_t kOrderCells = 32768;
+constexpr uint32_t kOrderWords = kOrderCells + 8 + 32;  // counts, box and barrier, slice totals
 
 // Device scratch owned by a scene (one per scene). The error word is sticky
 // (cleared by nlos_scene_check); the rest is reset by every forward pass.
 struct SceneScratch {
   unsigned int err;           // kErr* bits
   unsigned int pad;
-  // --- reset per pass from here ---
-  unsigned int peak_bits;     // max of tau_G as float bits (values are >= 0)
-  unsigned int pad2;
+  // --- reset per forward pass from here: its counters ---
   unsigned long long boundary_pairs;
-  double sum;                 // FP64 sum of tau_G over the cube
-  double sumsq;               // FP64 sum of squares
-  float scale;                // noise scale (computed on the device)
-  float dark;
   unsigned long long pairs_full;  // pairs through the full evaluation (past the early out)
   unsigned long long next_chunk;  // forward: next chunk of work units to claim
   unsigned long long pairs_tested;  // pairs of the units the forward staged
   unsigned long long n_live;      // forward: entries of its live-unit list
+  // --- reset by the detector as well from here: its results ---
+  unsigned int peak_bits;     // max of tau_G as float bits (values are >= 0)
+  unsigned int pad2;
+  double sum;                 // FP64 sum of tau_G over the cube
+  double sumsq;               // FP64 sum of squares
+  float scale;                // noise scale (computed on the device)
+  float dark;
+  unsigned long long deferred[2];  // header of the noise step's deferred-bin lists
 };
-constexpr size_t kScratchResetOffset = 8;  // offsetof(SceneScratch, peak_bits)
-static_assert(sizeof(SceneScratch) == 80, "scratch layout");
+constexpr size_t kScratchResetOffset = 8;    // offsetof(SceneScratch, boundary_pairs)
+constexpr size_t kScratchDetectOffset = 48;  // offsetof(SceneScratch, peak_bits)
+static_assert(sizeof(SceneScratch) == 96, "scratch layout");
 
 struct Geometry {
   // host-side resolved parameters; a scene may hold scan rows [row0, row0 + ny)
@@ -130,9 +134,12 @@ struct Geometry {
 
 struct SceneImpl;
 
-// Forward kernel launch (forward.cu). tau must be zeroed beforehand; the
-// kernel adds its (jittered, for NEAREST) partial histograms into it.
+// Forward launches (forward.cu) of a scene whose scratch counters are zero: tau
+// is zeroed, then the kernel adds its (jittered, for NEAREST) partial histograms.
 cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st);
+// The scene's forward plan (launch arguments, live-unit list), at its creation.
+cudaError_t forward_plan_create(SceneImpl& sc);
+void forward_plan_destroy(struct FwdPlan* p);
 cudaError_t launch_pair_table(const SceneImpl& sc, uint64_t s_begin, uint64_t s_count, float* u,
                               float* w, cudaStream_t st);
 // Adjoint (backward.cu).
@@ -162,7 +169,10 @@ cudaError_t launch_noise_scene(const float* tau, uint64_t n, SceneScratch* scrat
                                float peak_photons, float dark, float nr_db, uint64_t seed,
                                uint32_t stream_tag, uint32_t* counts, cudaStream_t st,
                                uint64_t index_base = 0, const double* cube_stats = nullptr,
-                               uint64_t cube_bins = 0);
+                               uint64_t cube_bins = 0, void* lists = nullptr);
+// Bytes of the deferred-bin lists that launch_noise_scene takes (their header
+// is scratch->deferred, zero at the launch); 0: none are used.
+size_t noise_list_bytes(uint64_t n, uint64_t index_base);
 cudaError_t launch_philox(const uint32_t* ctr, uint64_t n, uint32_t k0, uint32_t k1,
                           uint32_t* out, cudaStream_t st);
 
@@ -189,11 +199,13 @@ struct SceneImpl {
   float* base_points = nullptr;    // [P][8] records as given, once set_albedo_depth is used
   uint32_t* perm = nullptr;        // [P] packed position -> original point index
   uint16_t* cell = nullptr;        // [P] Morton cell of each point (ordering scratch)
-  uint32_t* cells = nullptr;       // [kOrderCells + 8] counts/cursors + box (ordering scratch)
+  uint32_t* cells = nullptr;       // [kOrderWords] counts/cursors, box, ... (ordering scratch)
   BlockBound* bounds = nullptr;    // [ceil(P / 2 / kSubPairs)]
   BlockBound* groups = nullptr;    // [ceil(P / 2 / kGroupPairs)]
   TileBound* tiles = nullptr;      // [ceil(S / kTile)] of scan_fwd
   OccSet occ{};                    // occluders (host copy; n = 0: none)
+  struct FwdPlan* fwd_plan = nullptr;  // (forward.cu; null without points)
+  void* noise_lists = nullptr;     // deferred-bin lists (detector.cu; noise_mode != NONE)
   cudaStream_t stream = nullptr;   // creation stream
   int device = 0;
   int num_sms = 0;
@@ -204,6 +216,7 @@ int jitter_radius(double sigma);
 // Spatial ordering, packing and block bounds of a scene's points (order.cu):
 // the device counting sort, then the pack and bounds kernels, on stream st.
 cudaError_t launch_order_pack(SceneImpl& s, cudaStream_t st);
+cudaError_t init_order(SceneImpl& s, cudaStream_t st);  // its scratch, once per scene
 // Tile bounds from a scan table (host).
 void tile_bounds_host(const ScanPoint* sp, uint64_t S, std::vector<TileBound>& out);
 

@@ -388,43 +388,62 @@ __global__ void __launch_bounds__(kDeferThreads) noise_deferred_kernel(const Noi
                         a.tag, rcp);
 }
 
-cudaError_t launch_noise_impl(const NoiseArgs& a, cudaStream_t st) {
+// Sizes of the deferred-bin lists: entries of the dense list, warp regions.
+uint64_t noise_cap(uint64_t n) { return std::min<uint64_t>(n, n / 32 + 4096); }
+uint64_t noise_groups_of(uint64_t n, uint64_t index_base) {
+  return ((index_base + n + 3) >> 2) - (index_base >> 2);
+}
+uint64_t noise_regions(uint64_t n, uint64_t index_base) {
+  return noise_groups_of(n, index_base) / 32 + 2;
+}
+
+size_t noise_list_bytes(uint64_t n, uint64_t index_base) {
+  if (!NLOS_NOISE_DEFER || n == 0 || n >= 0xFFFFFFFFull) return 0;
+  return noise_regions(n, index_base) * sizeof(unsigned long long) +
+         ((noise_cap(n) * sizeof(uint32_t) + 15) & ~(size_t)15);
+}
+
+cudaError_t launch_noise_impl(const NoiseArgs& a, cudaStream_t st, void* lists = nullptr) {
   if (a.n == 0) return cudaSuccess;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t groups = ((a.index_base + a.n + 3) >> 2) - (a.index_base >> 2);
+  const uint64_t groups = noise_groups_of(a.n, a.index_base);
   const uint64_t want = (groups + kNoiseThreads - 1) / kNoiseThreads;
   const uint64_t wave = (uint64_t)sms * kNoiseBlocksPerSm * NLOS_NOISE_WAVES;
   uint64_t blocks = want < wave ? want : wave;
   if (blocks > 1 && (blocks & 1u) == 0) --blocks;  // an odd number of warps (7 per block)
-  // the deferred-bin lists: the header, a dense list of local indices for
-  // about 3% of the bins, and one entry per warp region for the warps whose
-  // bins overflow it (the regions of 32 groups cover the launch's groups, plus
-  // one for an unaligned start); one stream-ordered allocation, freed after
-  // the second pass. Without it (or for parts of 2^32 - 1 bins or more) every
-  // bin is sampled in one pass.
+  // the deferred-bin lists: a dense list of local indices for about 3% of the
+  // bins, and one entry per warp region for the warps whose bins overflow it
+  // (the regions of 32 groups cover the launch's groups, plus one for an
+  // unaligned start). A scene keeps them (with their header in its scratch);
+  // elsewhere they are a stream-ordered allocation with the header in front,
+  // freed after the second pass. Without them (or for parts of 2^32 - 1 bins or
+  // more) every bin is sampled in one pass.
   NoiseArgs b = a;
   b.defer = DeferList{};
   cudaError_t e = cudaSuccess;
-  if (NLOS_NOISE_DEFER && a.n < 0xFFFFFFFFull) {
-    const uint64_t cap = std::min<uint64_t>(a.n, a.n / 32 + 4096);
-    const uint64_t n_reg = groups / 32 + 2;
-    const size_t bytes = 2 * sizeof(unsigned long long) + n_reg * sizeof(unsigned long long) +
-                         ((cap * sizeof(uint32_t) + 15) & ~(size_t)15);
-    void* buf = nullptr;
-    if (cudaMallocAsync(&buf, bytes, st) != cudaSuccess) {
+  void* buf = nullptr;
+  const size_t bytes = noise_list_bytes(a.n, a.index_base);
+  if (lists && bytes) {
+    b.defer.hdr = a.scratch->deferred;
+    b.defer.regions = static_cast<unsigned long long*>(lists);
+  } else if (bytes) {
+    const size_t hdr = 2 * sizeof(unsigned long long);
+    if (cudaMallocAsync(&buf, hdr + bytes, st) != cudaSuccess) {
+      buf = nullptr;
       (void)cudaGetLastError();  // no lists: one pass
-    } else if ((e = cudaMemsetAsync(buf, 0, 2 * sizeof(unsigned long long), st)) !=
-               cudaSuccess) {
+    } else if ((e = cudaMemsetAsync(buf, 0, hdr, st)) != cudaSuccess) {
       cudaFreeAsync(buf, st);
       return e;
     } else {
       b.defer.hdr = static_cast<unsigned long long*>(buf);
       b.defer.regions = b.defer.hdr + 2;
-      b.defer.bins = reinterpret_cast<uint32_t*>(b.defer.regions + n_reg);
-      b.defer.cap = (uint32_t)cap;
     }
+  }
+  if (b.defer.hdr) {
+    b.defer.bins = reinterpret_cast<uint32_t*>(b.defer.regions + noise_regions(a.n, a.index_base));
+    b.defer.cap = (uint32_t)noise_cap(a.n);
   }
   if (b.defer.hdr)
     noise_kernel<true><<<(unsigned)blocks, kNoiseThreads, 0, st>>>(b);
@@ -436,7 +455,9 @@ cudaError_t launch_noise_impl(const NoiseArgs& a, cudaStream_t st) {
       noise_deferred_kernel<<<(unsigned)(sms * 4), kDeferThreads, 0, st>>>(b);
       e = cudaGetLastError();
     }
-    const cudaError_t ef = cudaFreeAsync(b.defer.hdr, st);
+  }
+  if (buf) {
+    const cudaError_t ef = cudaFreeAsync(buf, st);
     if (e == cudaSuccess) e = ef;
   }
   return e;
@@ -461,7 +482,7 @@ cudaError_t launch_noise_scene(const float* tau, uint64_t n, SceneScratch* scrat
                                float peak_photons, float dark, float nr_db, uint64_t seed,
                                uint32_t tag, uint32_t* counts, cudaStream_t st,
                                uint64_t index_base, const double* cube_stats,
-                               uint64_t cube_bins) {
+                               uint64_t cube_bins, void* lists) {
   NoiseArgs a{};
   a.tau = tau;
   a.counts = counts;
@@ -476,7 +497,7 @@ cudaError_t launch_noise_scene(const float* tau, uint64_t n, SceneScratch* scrat
   a.peak_photons = peak_photons;
   a.dark_cfg = dark;
   a.nr_db = nr_db;
-  return launch_noise_impl(a, st);
+  return launch_noise_impl(a, st, lists);
 }
 
 // ---------------------------------------------------------------------------

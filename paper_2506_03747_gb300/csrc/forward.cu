@@ -59,18 +59,29 @@ __global__ void __launch_bounds__(1024, 1)
   if ((threadIdx.x & 31) == 0 && cnt.tested) atomicAdd(a.pairs_tested, cnt.tested * 64ull);
 }
 
+// Zeroes n floats from a 16-byte aligned p, by the whole grid.
+__device__ __forceinline__ void zero_floats(float* p, size_t n) {
+  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+  float4* p4 = reinterpret_cast<float4*>(p);
+  for (size_t i = t; i < n / 4; i += nt) p4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (size_t i = n / 4 * 4 + t; i < n; i += nt) p[i] = 0.f;
+}
+
 // The live units of a pass, for the forward's chunk claims: one CTA per
 // (tile, window) tests the point blocks against the bounds (unit_live, as
 // the producer warp would) and appends the live ones, with the histogram rows
 // they can touch, to the list (unit | rows << 32). Entries of one (tile,
 // window) are contiguous, so a chunk of the list rarely spans two tiles; the
-// order of the (tile, window) runs in the list does not matter.
+// order of the (tile, window) runs in the list does not matter. The same launch
+// zeroes the output that the forward adds to.
 template <int SCAN, int COS, int MODE>
 __global__ void __launch_bounds__(256) unit_list_kernel(const __grid_constant__ FwdArgs a,
                                                         unsigned long long* __restrict__ list,
                                                         unsigned long long* __restrict__ n_live) {
   __shared__ uint32_t s_warp[8];
   __shared__ unsigned long long s_base;
+  zero_floats(a.tau, (size_t)a.S * a.B);
+  if (MODE == MODE_SPLAT_MOM) zero_floats(a.far_mass, a.S);
   const unsigned long long tw = blockIdx.x;
   const float margin = window_margin<MODE>(a);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -274,15 +285,79 @@ int jitter_radius(double sigma) {
   return (int)std::ceil(2.0 * sigma);
 }
 
-cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
-  const Geometry& g = sc.g;
-  cudaError_t e = cudaMemsetAsync(tau, 0, sizeof(float) * g.S * g.B, st);
-  if (e != cudaSuccess || g.P == 0 || g.S == 0) return e;
-
+// What every forward of a scene takes, resolved once: the launch's arguments
+// and shape, and the live-unit list's memory (resolving it on each call, with a
+// list from the stream-ordered pool and three memsets, made the smallest scene's
+// pass 32 us of host calls). Only occluders change it (the kernel's mode).
+struct FwdPlan {
   FwdArgs a{};
+  MomTab mt{};
+  int mode = -1;
+  FwdFn fn = nullptr;
+  ListFn list_fn = nullptr;  // null: chunks of all units are claimed
+  size_t smem = 0;
+  unsigned grid = 0;
+  unsigned long long* list = nullptr;  // [units], or null
+};
+
+namespace {
+
+int forward_mode(const SceneImpl& sc) {
+  const Geometry& g = sc.g;
+  return g.bin_mode == NLOS_BIN_SPLAT ? (use_moments(g.sigma) ? MODE_SPLAT_MOM : MODE_SPLAT)
+         : sc.params.boundary_eps > 0.f ? MODE_NEAREST_COUNT
+         : sc.occ.n > 0                 ? MODE_NEAREST_OCC
+                                        : MODE_NEAREST;
+}
+
+// Kernels of the plan's mode, allowed all of the shared memory an SM has.
+cudaError_t plan_mode(FwdPlan& p, const SceneImpl& sc, int mode) {
+  const Geometry& g = sc.g;
+  p.mode = mode;
+  p.fn = pick(g.scan_mode, g.cos_mode, mode);
+  p.list_fn = p.list ? pick_list(g.scan_mode, g.cos_mode, mode) : nullptr;
+  int optin = 0, per_sm = 0;
+  cudaFuncAttributes fa{};
+  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, sc.device);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, p.fn);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             optin - (int)fa.sharedSizeBytes);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, p.fn, 1024, p.smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  p.grid = (unsigned)std::min<unsigned long long>((unsigned long long)sc.num_sms * per_sm, p.a.units);
+  // chunks of units claimed by the CTAs where there is no list: about
+  // NLOS_FWD_CHUNKS_PER_CTA per CTA, but at least 8 units (a chunk mostly ends
+  // in a tile change, whose flush is worth amortising) and at most 64 (finer
+  // claims even out the cost of units, which the bounds do not predict), and
+  // never so large that some CTA would get none. Measured on the union (32768
+  // units: 8 beats 6.7 per chunk) and heightfield (524288 units: 64 beats 108).
+  const unsigned long long per_cta =
+      p.a.units / ((unsigned long long)p.grid * NLOS_FWD_CHUNKS_PER_CTA);
+  p.a.chunk = std::min<unsigned long long>(
+      std::min<unsigned long long>(std::max<unsigned long long>(per_cta, 8), 64),
+      std::max<unsigned long long>(1, p.a.units / p.grid));
+  return cudaSuccess;
+}
+
+}  // namespace
+
+void forward_plan_destroy(FwdPlan* p) {
+  if (!p) return;
+  if (p->list) cudaFree(p->list);
+  if (p->a.far_mass) cudaFree(p->a.far_mass);
+  delete p;
+}
+
+cudaError_t forward_plan_create(SceneImpl& sc) {
+  const Geometry& g = sc.g;
+  if (g.P == 0 || g.S == 0) return cudaSuccess;
+  FwdPlan* p = sc.fwd_plan = new FwdPlan();
+  FwdArgs& a = p->a;
   a.pairs = sc.pairs;
   a.scan = sc.scan_fwd;
-  a.tau = tau;
   a.err = &sc.scratch->err;
   a.boundary = &sc.scratch->boundary_pairs;
   a.pairs_full = &sc.scratch->pairs_full;
@@ -295,17 +370,11 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
   a.S = (uint32_t)g.S;
   a.B = g.B;
   a.kbin = (float)((g.scan_mode == NLOS_CONFOCAL ? 2.0 : 1.0) / g.cdt);
-  const bool splat = g.bin_mode == NLOS_BIN_SPLAT;
-  MomTab mt{};
-  const bool moments = splat && use_moments(g.sigma);
-  const int mode = moments ? MODE_SPLAT_MOM
-                   : splat ? MODE_SPLAT
-                   : sc.params.boundary_eps > 0.f ? MODE_NEAREST_COUNT
-                   : sc.occ.n > 0 ? MODE_NEAREST_OCC
-                                  : MODE_NEAREST;
-  if (moments) moment_table(g.sigma, mt);
+  const int mode = forward_mode(sc);
+  const bool moments = mode == MODE_SPLAT_MOM;
+  if (moments) moment_table(g.sigma, p->mt);
   a.eps = sc.params.boundary_eps;
-  if (splat) {
+  if (g.bin_mode == NLOS_BIN_SPLAT) {
     const double s = g.sigma;
     a.inv2s2 = (float)(1.0 / (2.0 * s * s));
     a.norm = (float)(1.0 / (s * std::sqrt(2.0 * 3.14159265358979323846)));
@@ -320,11 +389,12 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
     if (a.replicate) jitter_tails(a.taps, a.R, a.tail);
   }
 
-  // shared memory: histogram [bw][32] floats + two staged blocks + barriers
-  int dev = sc.device, optin = 0;
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // shared memory: histogram [bw][32] floats + the staged slots + barriers
+  int optin = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, sc.device);
+  if (e != cudaSuccess) return e;
   // pairs per staged block: NLOS_FWD_PPB, halved while the histogram of a
-  // full window (up to 1024 bins) would not fit beside the two stages
+  // full window (up to 1024 bins) would not fit beside the stages
   a.ppb = NLOS_FWD_PPB;
   a.stages = NLOS_FWD_STAGES;
   while (a.ppb > 256 && (size_t)std::min(g.B, 1024u) * kTile * 4 +
@@ -335,98 +405,88 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
     a.ppb = kPairsPerBlock;
     a.stages = 2;
   }
-  // staged blocks, then full + empty barriers and the unit number of each slot
-  const size_t stage_bytes = a.stages * (size_t)a.ppb * sizeof(PointPair) + 24 * a.stages + 64 +
-                             8 * 32 + 4 * kRowWords + 4 * kMaxRangedStages;
-  size_t smem;
+  const uint32_t n_tiles = (uint32_t)((g.S + kTile - 1) / kTile);
+  // staged blocks, then full + empty barriers and what each slot holds
+  auto stage_bytes = [&]() {
+    return a.stages * (size_t)a.ppb * sizeof(PointPair) + 24 * a.stages + 64 + 8 * 32 +
+           4 * kRowWords + 4 * kMaxRangedStages;
+  };
   if (moments) {
     // windows of at most kMomRows rows over the bins and J beyond each end
-    a.halo = mt.J;
-    const uint32_t max_bw = (uint32_t)(kMomRows / mt.q), bins = g.B + 2u * (uint32_t)a.halo;
+    a.halo = p->mt.J;
+    const uint32_t max_bw = (uint32_t)(kMomRows / p->mt.q), bins = g.B + 2u * (uint32_t)p->mt.J;
     a.n_win = (bins + max_bw - 1) / max_bw;
     a.bw = (bins + a.n_win - 1) / a.n_win;
-    smem = (size_t)kMoments * kMomRows * kTile * 4 + stage_bytes;
   } else {
-    uint32_t max_bw = (uint32_t)(((size_t)optin - stage_bytes) / (kTile * 4)) & ~3u;
+    const uint32_t max_bw = (uint32_t)(((size_t)optin - stage_bytes()) / (kTile * 4)) & ~3u;
     a.n_win = (g.B + max_bw - 1) / max_bw;
     a.bw = ((g.B + a.n_win - 1) / a.n_win + 3) & ~3u;
-    smem = (size_t)a.bw * kTile * 4 + stage_bytes;
   }
-  const uint32_t n_tiles = (uint32_t)((g.S + kTile - 1) / kTile);
+  // a scene of few units is cut into smaller blocks, so that more SMs take part
+  // (the 32 x 32 scan of 1,024 points has 32 units of 1,024: 32.1 us a pass in one
+  // block, 22 us in blocks of 128 points)
+  while (a.ppb > kFwdMinPpb && n_tiles * a.n_win * ((a.n_pairs + a.ppb - 1) / a.ppb) <
+                                   (uint64_t)sc.num_sms)
+    a.ppb /= 2;
+  p->smem = (moments ? (size_t)kMoments * kMomRows : (size_t)a.bw) * kTile * 4 + stage_bytes();
   a.n_blk = (a.n_pairs + a.ppb - 1) / a.ppb;
   a.units = (unsigned long long)n_tiles * a.n_win * a.n_blk;
-
-  FwdFn fn = pick(g.scan_mode, g.cos_mode, mode);
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  // 1024 threads when only one CTA fits on an SM, else 512 (register budget)
-  int threads = 512, per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm <= 1 || NLOS_FWD_ONE_CTA) {
-    threads = 1024;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
-    if (e != cudaSuccess) return e;
+  if (moments) {
+    e = cudaMalloc(reinterpret_cast<void**>(&a.far_mass), sizeof(float) * g.S);
+    if (e != cudaSuccess) {
+      a.far_mass = nullptr;
+      return e;
+    }
   }
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  unsigned long long grid = (unsigned long long)sc.num_sms * per_sm;
-  if (grid > a.units) grid = a.units;
-  // chunks of units claimed by the CTAs: about NLOS_FWD_CHUNKS_PER_CTA per
-  // CTA, but at least 8 units (a chunk mostly ends in a tile change, whose
-  // flush is worth amortising) and at most 64 (finer claims even out the
-  // cost of units, which the bounds do not predict), and never so large that
-  // some CTA would get none. Measured on the union (32768 units: 8 beats
-  // 6.7 per chunk) and heightfield (524288 units: 64 beats 108) workloads.
-  const unsigned long long per_cta = a.units / (grid * NLOS_FWD_CHUNKS_PER_CTA);
-  a.chunk = std::min<unsigned long long>(std::min<unsigned long long>(std::max<unsigned long long>(per_cta, 8), 64),
-                                         std::max<unsigned long long>(1, a.units / grid));
   // With block bounds, a first kernel lists the live units and the forward
   // claims chunks of that list: a chunk then holds NLOS_FWD_LIST_MIN.. units
   // that all carry work (mostly of one tile), instead of a fixed run of
   // units of which most may be culled, so tile changes (flush, zeroing,
-  // barriers) are fewer per unit of work.
-  ListFn lf = (NLOS_FWD_CULL && a.bounds) ? pick_list(g.scan_mode, g.cos_mode, mode) : nullptr;
-  unsigned long long* list = nullptr;
-  if (lf) {
-    // the moment form's far_mass lies behind the list
-    const size_t list_bytes = sizeof(unsigned long long) * a.units;
-    e = cudaMallocAsync(reinterpret_cast<void**>(&list),
-                        list_bytes + (moments ? sizeof(float) * g.S : 0), st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(&sc.scratch->n_live, 0, sizeof(unsigned long long), st);
-    if (moments && e == cudaSuccess) {
-      a.far_mass = reinterpret_cast<float*>(list + a.units);
-      e = cudaMemsetAsync(a.far_mass, 0, sizeof(float) * g.S, st);
-    }
-    if (e == cudaSuccess) {
-      lf<<<(unsigned)(a.units / a.n_blk), 256, 0, st>>>(a, list, &sc.scratch->n_live);
-      e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) {
-      cudaFreeAsync(list, st);
-      return e;
-    }
-    a.unit_list = list;
-    a.n_live = &sc.scratch->n_live;
-    a.list_chunks_per_cta = NLOS_FWD_LIST_CHUNKS_PER_CTA;
-    a.list_min_chunk = NLOS_FWD_LIST_MIN;
-    a.list_max_chunk = NLOS_FWD_LIST_MAX;
-    // a moment flush costs as much as several units, so its list goes out in
-    // one range per CTA (static 60 / 85 / 100%: 0.72 / 0.69 / 0.66 ms on the
-    // 64 x 64 scan of 65,536 points at sigma = 3.2, 0.17 / 0.19 / 0.13 ms on the 32 x 32
-    // scan of 16,384 points at sigma = 1.6)
-    a.list_static_pct = moments ? NLOS_FWD_MOM_STATIC : NLOS_FWD_LIST_STATIC;
+  // barriers) are fewer per unit of work. Without memory for it the producers
+  // test the units themselves.
+  if (NLOS_FWD_CULL && mode != MODE_NEAREST_COUNT &&
+      cudaMalloc(reinterpret_cast<void**>(&p->list), sizeof(unsigned long long) * a.units) !=
+          cudaSuccess) {
+    p->list = nullptr;
+    (void)cudaGetLastError();
   }
-  fn<<<(unsigned)grid, threads, smem, st>>>(a, mt, sc.occ);
-  e = cudaGetLastError();
-  if (moments && e == cudaSuccess) {
+  a.unit_list = p->list;
+  a.n_live = &sc.scratch->n_live;
+  a.list_chunks_per_cta = NLOS_FWD_LIST_CHUNKS_PER_CTA;
+  a.list_min_chunk = NLOS_FWD_LIST_MIN;
+  a.list_max_chunk = NLOS_FWD_LIST_MAX;
+  // a moment flush costs as much as several units, so its list goes out in
+  // one range per CTA (static 60 / 85 / 100%: 0.72 / 0.69 / 0.66 ms on the
+  // 64 x 64 scan of 65,536 points at sigma = 3.2, 0.17 / 0.19 / 0.13 ms on the 32 x 32
+  // scan of 16,384 points at sigma = 1.6)
+  a.list_static_pct = moments ? NLOS_FWD_MOM_STATIC : NLOS_FWD_LIST_STATIC;
+  return plan_mode(*p, sc, mode);
+}
+
+cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
+  const Geometry& g = sc.g;
+  FwdPlan* p = sc.fwd_plan;
+  cudaError_t e = cudaSuccess;
+  if (p && p->mode != forward_mode(sc) &&
+      (e = plan_mode(*p, sc, forward_mode(sc))) != cudaSuccess)
+    return e;
+  if (!p || !p->list_fn) e = cudaMemsetAsync(tau, 0, sizeof(float) * g.S * g.B, st);
+  if (p && !p->list_fn && p->a.far_mass && e == cudaSuccess)
+    e = cudaMemsetAsync(p->a.far_mass, 0, sizeof(float) * g.S, st);
+  if (e != cudaSuccess || !p) return e;
+  FwdArgs a = p->a;
+  a.tau = tau;
+  if (p->list_fn) {
+    // (the counters, n_live among them, were zeroed with the pass's scratch)
+    p->list_fn<<<(unsigned)(a.units / a.n_blk), 256, 0, st>>>(a, p->list, &sc.scratch->n_live);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  p->fn<<<p->grid, 1024, p->smem, st>>>(a, p->mt, sc.occ);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (p->mode == MODE_SPLAT_MOM) {
     const unsigned blocks = (unsigned)std::min<uint64_t>((g.S + 7) / 8, (uint64_t)sc.num_sms * 8);
     pick_tail(g.scan_mode, g.cos_mode)<<<blocks, 256, 0, st>>>(a);
     e = cudaGetLastError();
-  }
-  if (list) {
-    const cudaError_t ef = cudaFreeAsync(list, st);
-    if (e == cudaSuccess) e = ef;
   }
   return e;
 }

@@ -35,9 +35,6 @@ constexpr int kPairsPerBlock = 256;         // serving kernel: 16 KB per staged 
 #ifndef NLOS_FWD_PPB
 #define NLOS_FWD_PPB 512                    // standalone forward: pairs per staged block
 #endif
-#ifndef NLOS_FWD_ONE_CTA
-#define NLOS_FWD_ONE_CTA 1                  // standalone forward: 1 CTA x 1024 threads per SM
-#endif
 #ifndef NLOS_FWD_SQRT_RCP
 #define NLOS_FWD_SQRT_RCP 1                 // r from sqrt.approx, weights from one rcp.approx
 #endif
@@ -75,6 +72,7 @@ constexpr int kPairsPerBlock = 256;         // serving kernel: 16 KB per staged 
 #define NLOS_FWD_UNROLL 4                   // standalone forward: unroll of the pair loop
 #endif
 
+constexpr uint32_t kFwdMinPpb = 64;  // smallest block of a scene of few units
 constexpr int kFwdUnroll = NLOS_FWD_UNROLL;  // (#pragma unroll takes no macro)
 
 enum { MODE_NEAREST = 0, MODE_NEAREST_COUNT = 1, MODE_SPLAT = 2, MODE_SPLAT_MOM = 3,
@@ -821,8 +819,8 @@ __device__ __forceinline__ float imax(float a0, float a1, float b0, float b1) {
 // weight. Conservative: a unit it keeps may still bin nothing.
 // Bounds of point block blk: the union of its sub-blocks' bounds.
 __device__ __forceinline__ BlockBound block_bound(const FwdArgs& a, uint32_t blk) {
-  const uint32_t sub_per = a.ppb / kSubPairs;
-  const uint32_t sb0 = blk * sub_per;
+  const uint32_t sub_per = max(1u, a.ppb / kSubPairs);
+  const uint32_t sb0 = blk * a.ppb / kSubPairs;  // (a block smaller than a sub-block lies in one)
   const uint32_t n_sub = (a.n_pairs + kSubPairs - 1) / kSubPairs;
   BlockBound b = a.bounds[sb0];
   for (uint32_t j = 1; j < sub_per && sb0 + j < n_sub; ++j) {

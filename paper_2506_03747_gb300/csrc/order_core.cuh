@@ -137,47 +137,35 @@ __device__ __forceinline__ void cell_range(const float* __restrict__ raw, uint64
   }
 }
 
+// Inclusive prefix sum over a warp.
+__device__ __forceinline__ uint32_t inclusive_scan(uint32_t x) {
+  const int lane = threadIdx.x & 31;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
 // counts[c] <- sum of counts[0..c). One CTA of exactly 1024 threads: warp w
 // scans cells [w * 1024, (w + 1) * 1024) 32 at a time (coalesced loads,
 // shuffle scans), then the 32 warp totals are scanned; wsum: 32 shared words.
-// PREFETCH loads a warp's 1024 counts into registers before the serial
-// carry chain (32 loads in flight instead of one at a time; 32 registers).
-template <bool PREFETCH = false>
 __device__ __forceinline__ void scan_cells(uint32_t* counts, uint32_t* wsum) {
   constexpr int kPerWarp = kOrderCells / 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t* seg = counts + (size_t)w * kPerWarp;
-  uint32_t pre[PREFETCH ? kPerWarp / 32 : 1];
-  if (PREFETCH) {
-#pragma unroll
-    for (int j = 0; j < kPerWarp / 32; ++j) pre[j] = seg[32 * j + lane];
-  }
   uint32_t carry = 0;
-  auto step = [&](int j, uint32_t v) {
-    uint32_t x = v;  // inclusive scan of the 32 values
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
+  for (int j = 0; j < kPerWarp; j += 32) {
+    const uint32_t v = seg[j + lane];
+    const uint32_t x = inclusive_scan(v);
     seg[j + lane] = carry + x - v;  // exclusive within the warp's segment
     carry += __shfl_sync(0xffffffffu, x, 31);
-  };
-  if (PREFETCH) {
-#pragma unroll
-    for (int j = 0; j < kPerWarp; j += 32) step(j, pre[j / 32]);
-  } else {
-    for (int j = 0; j < kPerWarp; j += 32) step(j, seg[j + lane]);
   }
   if (lane == 0) wsum[w] = carry;
   __syncthreads();
   if (w == 0) {
     const uint32_t v = wsum[lane];
-    uint32_t x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    wsum[lane] = x - v;
+    wsum[lane] = inclusive_scan(v) - v;
   }
   __syncthreads();
   const uint32_t base = wsum[w];
@@ -185,19 +173,24 @@ __device__ __forceinline__ void scan_cells(uint32_t* counts, uint32_t* wsum) {
   __syncthreads();
 }
 
+// The lanes of one cell take consecutive slots from one atomic on its cursor.
+// base (nullable): added to the cursors of each kSliceCells cells.
+constexpr uint32_t kSliceCells = 1024;
 __device__ __forceinline__ void scatter_range(const uint16_t* cell, uint64_t b, uint64_t e,
                                               uint64_t t0, uint64_t stride, uint32_t* cursor,
-                                              uint32_t* perm) {
+                                              uint32_t* perm, const uint32_t* base_of = nullptr,
+                                              uint64_t limit = ~0ull) {
   const uint32_t lane = threadIdx.x & 31;
   for (uint64_t i = b + t0; i < e; i += stride) {
     const uint32_t k = cell[i];
-    // the lanes of one cell take consecutive slots from one atomic
     const unsigned peers = __match_any_sync(__activemask(), k);
     const int leader = __ffs(peers) - 1;
     uint32_t base = 0;
     if ((int)lane == leader) base = atomicAdd(&cursor[k], (uint32_t)__popc(peers));
     base = __shfl_sync(peers, base, leader);
-    perm[base + (uint32_t)__popc(peers & ((1u << lane) - 1u))] = (uint32_t)i;
+    const uint32_t slot = base + (uint32_t)__popc(peers & ((1u << lane) - 1u)) +
+                          (base_of ? base_of[k / kSliceCells] : 0u);
+    if (slot < limit) perm[slot] = (uint32_t)i;
   }
 }
 

@@ -164,6 +164,8 @@ nlos_status scene_create_rows(const nlos_params* params, const float* pts, uint6
                     (void*)s.perm, (void*)s.cell, (void*)s.cells, (void*)s.bounds, (void*)s.groups,
                     (void*)s.tiles})
       if (q) cudaFree(q);
+    if (s.noise_lists) cudaFree(s.noise_lists);
+    forward_plan_destroy(s.fwd_plan);
     delete sc;
     return set_error(code, msg);
   };
@@ -186,12 +188,23 @@ nlos_status scene_create_rows(const nlos_params* params, const float* pts, uint6
       (P > 0 && (e = cudaMalloc(&s.raw_points, sizeof(float) * 8 * P)) != cudaSuccess) ||
       (P > 0 && (e = cudaMalloc(&s.perm, sizeof(uint32_t) * P)) != cudaSuccess) ||
       (P > 0 && (e = cudaMalloc(&s.cell, sizeof(uint16_t) * P)) != cudaSuccess) ||
-      (P > 0 && (e = cudaMalloc(&s.cells, sizeof(uint32_t) * (kOrderCells + 8))) != cudaSuccess) ||
+      (P > 0 && (e = cudaMalloc(&s.cells, sizeof(uint32_t) * kOrderWords)) != cudaSuccess) ||
       (P > 0 && (e = cudaMalloc(&s.bounds, sizeof(BlockBound) * n_sub)) != cudaSuccess) ||
       (P > 0 && (e = cudaMalloc(&s.groups, sizeof(BlockBound) *
                                                ((n_pairs + kGroupPairs - 1) / kGroupPairs))) !=
                     cudaSuccess))
     return fail(NLOS_ENOMEM, std::string("device allocation failed: ") + cudaGetErrorString(e));
+
+  const size_t list_bytes =
+      g.noise_mode != NLOS_NOISE_NONE ? noise_list_bytes(g.S * g.B, (uint64_t)g.row0 * g.nx * g.B) : 0;
+  // (without lists of its own the scene's noise step takes them from the pool)
+  if (list_bytes && cudaMalloc(&s.noise_lists, list_bytes) != cudaSuccess) {
+    s.noise_lists = nullptr;
+    (void)cudaGetLastError();
+  }
+  if ((e = forward_plan_create(s)) != cudaSuccess)
+    return fail(e == cudaErrorMemoryAllocation ? NLOS_ENOMEM : NLOS_ECUDA,
+                std::string("forward plan: ") + cudaGetErrorString(e));
 
   e = cudaMemsetAsync(s.scratch, 0, sizeof(SceneScratch), st);
   if (e == cudaSuccess)
@@ -203,6 +216,7 @@ nlos_status scene_create_rows(const nlos_params* params, const float* pts, uint6
   if (e == cudaSuccess && P > 0)
     e = cudaMemcpyAsync(s.raw_points, pts, sizeof(float) * 8 * P,
                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && P > 0) e = init_order(s, st);
   if (e == cudaSuccess && P > 0) e = launch_order_pack(s, st);
   unsigned int err = 0;
   if (e == cudaSuccess)
@@ -309,6 +323,8 @@ nlos_status scene_destroy(nlos_scene* sc) {
   for (void* q : {(void*)s.perm, (void*)s.cell, (void*)s.cells, (void*)s.bounds, (void*)s.groups,
                     (void*)s.tiles})
     if (q && (e2 = cudaFree(q)) != cudaSuccess) e = e2;
+  if (s.noise_lists && (e2 = cudaFree(s.noise_lists)) != cudaSuccess) e = e2;
+  forward_plan_destroy(s.fwd_plan);
   delete sc;
   if (e != cudaSuccess) return cuda_error(e, "cudaFree");
   return NLOS_OK;
