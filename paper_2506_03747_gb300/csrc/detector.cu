@@ -308,16 +308,17 @@ struct NoiseArgs {
 // indices, and a stride that is a multiple of the bin count (a wave of
 // 256-thread blocks of 1024-bin transients: 1216 * 256 = 304 * 1024) gave some
 // warps every bright bin of the cube (ncu: SMs 40% active, ALU pipe from 19%
-// to 99% over the SMs). With up to 16 waves a thread mostly takes one group,
-// and the CTAs that meet bright bins are the ones that run long (heightfield128
-// 0.139 ms against 0.156 ms with one wave and a longer stride loop; union64
-// 0.060 against 0.057). No atomics and no divisions in the loop; 1/k of the
-// inversion search from a shared table.
+// to 99% over the SMs). A few waves of short CTAs balance the bright bins (16,384
+// x 1,024 bins, mean 1 count: 2 / 4 / 16 waves 103.8 / 102.1 / 102.8 us of
+// detector, and 69.7 / 67.0 / 72.3 us at a twentieth of the light). No atomics and
+// no divisions in the loop. Bound: ALU issue; that detector took 140.6 us with a
+// 13-instruction search step, an integer conversion a bin and tables of 1/k that
+// each short CTA filled.
 constexpr int kNoiseWarps = 7;
 constexpr int kNoiseThreads = 32 * kNoiseWarps;
 constexpr int kNoiseBlocksPerSm = 8;
 #ifndef NLOS_NOISE_WAVES
-#define NLOS_NOISE_WAVES 16  // resident waves of CTAs at most (the rest by the grid stride)
+#define NLOS_NOISE_WAVES 4   // resident waves of CTAs at most (the rest by the grid stride)
 #endif
 
 #ifndef NLOS_NOISE_DEFER
@@ -341,11 +342,6 @@ __device__ __forceinline__ void launch_scale(const NoiseArgs& a, float& scale, f
 
 template <bool DEFER>
 __global__ void __launch_bounds__(kNoiseThreads, kNoiseBlocksPerSm) noise_kernel(const NoiseArgs a) {
-  // one table per warp, so that no CTA barrier is needed (CTAs are short)
-  __shared__ float rcp_tab[kNoiseWarps][kRcpTable];
-  float* rcp = rcp_tab[threadIdx.x >> 5];
-  fill_rcp_table(rcp, threadIdx.x & 31, 32);
-  __syncwarp();
   float scale, dark;
   launch_scale(a, scale, dark);
   if (a.scratch && blockIdx.x == 0 && threadIdx.x == 0) {
@@ -355,7 +351,7 @@ __global__ void __launch_bounds__(kNoiseThreads, kNoiseBlocksPerSm) noise_kernel
   const uint64_t stride = (uint64_t)gridDim.x * kNoiseWarps * 32;
   const uint64_t j0 = ((uint64_t)blockIdx.x * kNoiseWarps + (threadIdx.x >> 5)) * 32 +
                       (threadIdx.x & 31);
-  noise_groups<DEFER>(a.tau, a.counts, 0, a.n, a.index_base, scale, dark, a.seed, a.tag, rcp, j0,
+  noise_groups<DEFER>(a.tau, a.counts, 0, a.n, a.index_base, scale, dark, a.seed, a.tag, j0,
                       stride, &a.defer);
 }
 
@@ -365,10 +361,6 @@ __global__ void __launch_bounds__(kNoiseThreads, kNoiseBlocksPerSm) noise_kernel
 constexpr int kDeferThreads = 256;
 
 __global__ void __launch_bounds__(kDeferThreads) noise_deferred_kernel(const NoiseArgs a) {
-  __shared__ float rcp_tab[kDeferThreads / 32][kRcpTable];  // one table per warp
-  float* rcp = rcp_tab[threadIdx.x >> 5];
-  fill_rcp_table(rcp, threadIdx.x & 31, 32);
-  __syncwarp();
   float scale, dark;
   launch_scale(a, scale, dark);
   const DeferList& d = a.defer;
@@ -378,14 +370,14 @@ __global__ void __launch_bounds__(kDeferThreads) noise_deferred_kernel(const Noi
   for (uint64_t k = (uint64_t)blockIdx.x * kDeferThreads + threadIdx.x; k < nd; k += nt) {
     const uint32_t l = d.bins[k];
     if (l != kDeferredCount)
-      noise_deferred_bin(a.tau, a.counts, l, a.index_base, scale, dark, a.seed, a.tag, rcp);
+      noise_deferred_bin(a.tau, a.counts, l, a.index_base, scale, dark, a.seed, a.tag);
   }
   const unsigned long long nr = *(volatile unsigned long long*)&d.hdr[1];
   const uint64_t nw = nt / 32;
   for (uint64_t k = (uint64_t)blockIdx.x * (kDeferThreads / 32) + (threadIdx.x >> 5); k < nr;
        k += nw)
     noise_deferred_warp(a.tau, a.counts, a.n, d.regions[k], a.index_base, scale, dark, a.seed,
-                        a.tag, rcp);
+                        a.tag);
 }
 
 // Sizes of the deferred-bin lists: entries of the dense list, warp regions.

@@ -34,10 +34,24 @@ namespace nlos {
 // multiply-adds, where Knuth's product method takes about lambda uniforms.
 constexpr float kInvMax = 30.0f;
 constexpr float kSplitMax = 150.0f;
-constexpr int kRcpTable = 64;  // 1/k for k < kRcpTable from a table (shared memory)
+// 1/k rounded to single precision (as the host's 1.0f / k) for k < kRcpTable, in
+// constant memory: the lanes of a warp take the same step of their searches
+// together, so a step's read is one broadcast. (A table per warp in shared
+// memory had to be filled by every short-lived CTA.)
+constexpr int kRcpTable = 128;
+struct RcpTable {
+  float v[kRcpTable];
+  constexpr RcpTable() : v() {
+    for (int k = 1; k < kRcpTable; ++k) v[k] = 1.0f / (float)k;
+  }
+};
+static __constant__ constexpr RcpTable c_rcp{};
 
+// ((w >> 9) + 0.5) 2^-23. The 23 bits go into the mantissa of 2^23 + m, from which
+// m + 0.5 is one exact subtraction (an integer conversion takes the quarter-rate
+// pipe).
 __device__ __forceinline__ float word_uniform(uint32_t w) {
-  return __fmul_rn(__fadd_rn((float)(w >> 9), 0.5f), 0x1p-23f);
+  return __fmul_rn(__fadd_rn(__uint_as_float(0x4B000000u | (w >> 9)), -8388607.5f), 0x1p-23f);
 }
 
 // The Philox block of group g (the first draws of bins 4g .. 4g + 3).
@@ -74,24 +88,62 @@ struct BinStream {
   }
 };
 
-// 1/k rounded to single precision (the correctly rounded reciprocal, as the
-// host's 1.0f / k); rcp: a table of kRcpTable entries or null.
-__device__ __forceinline__ float recip_k(uint32_t k, const float* rcp) {
-  return (rcp && k < (uint32_t)kRcpTable) ? rcp[k] : __frcp_rn((float)k);
-}
-
-__device__ __forceinline__ uint32_t poisson_inversion(float lam, float u, const float* rcp) {
-  float p = expf(-lam);
-  float F = p;
-  uint32_t k = 0;
+// The search from term k on, without a table (the last term p, sum F).
+__device__ __forceinline__ uint32_t inversion_tail(float lam, float u, float p, float F,
+                                                       uint32_t k) {
   while (u > F && k < 1000u) {
     k += 1u;
-    p = __fmul_rn(__fmul_rn(p, lam), recip_k(k, rcp));
+    p = __fmul_rn(__fmul_rn(p, lam), __frcp_rn((float)k));
     const float Fn = __fadd_rn(F, p);
     if (Fn == F) break;
     F = Fn;
   }
   return k;
+}
+
+// A warp takes as many steps as its brightest bin, so the step is what the
+// kernel costs: seven instructions with the steps unrolled and one exit test
+// (with bounds on k and a table lookup by index: thirteen).
+__device__ __forceinline__ uint32_t poisson_inversion(float lam, float u) {
+  float p = expf(-lam);
+  float F = p;
+  if (!(u > F)) return 0u;
+  uint32_t k = 0;
+#pragma unroll 1
+  for (; k < (uint32_t)kRcpTable - 4u; k += 4) {
+#pragma unroll
+    for (uint32_t j = 1; j <= 4; ++j) {
+      p = __fmul_rn(__fmul_rn(p, lam), c_rcp.v[k + j]);
+      const float Fn = __fadd_rn(F, p);
+      if (Fn == F || !(u > Fn)) return k + j;
+      F = Fn;
+    }
+  }
+  return inversion_tail(lam, u, p, F, k);
+}
+
+// The sum of the first `parts` (2 to 5) inversion draws of mean lam with
+// uniforms u[0 .. parts): the draws share one walk along the terms, each step
+// adding one for every draw that is still below its uniform.
+__device__ __forceinline__ uint32_t poisson_inversions(float lam, const float u[5], int parts) {
+  float v[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) v[i] = i < parts ? u[i] : -1.0f;  // never above F
+  float p = expf(-lam);
+  float F = p;
+  uint32_t total = 0;
+  for (uint32_t k = 1; k <= 1000u; ++k) {
+    uint32_t c = 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) c += v[i] > F ? 1u : 0u;
+    if (c == 0u) break;
+    total += c;
+    p = __fmul_rn(__fmul_rn(p, lam), k < (uint32_t)kRcpTable ? c_rcp.v[k] : __frcp_rn((float)k));
+    const float Fn = __fadd_rn(F, p);
+    if (Fn == F) break;
+    F = Fn;
+  }
+  return total;
 }
 
 __device__ __forceinline__ uint32_t poisson_ptrs(float lam_f, BinStream& st) {
@@ -122,40 +174,35 @@ __device__ __forceinline__ uint32_t poisson_ptrs(float lam_f, BinStream& st) {
 // lambda >= 30, out of line: these bins are rare (the bright bins of a
 // cube), and inlined their paths would set the register budget of every bin.
 static __device__ __noinline__ uint32_t poisson_large(float lam, float u0, uint64_t index,
-                                                      uint64_t seed, uint32_t tag,
-                                                      const float* rcp) {
-  BinStream st(index, seed, tag);
+                                                      uint64_t seed, uint32_t tag) {
   if (lam < kSplitMax) {
     const float parts = ceilf(__fdiv_rn(lam, kInvMax));
     const float sub = __fdiv_rn(lam, parts);
-    uint32_t k = poisson_inversion(sub, u0, rcp);
-    for (int i = 1; i < (int)parts; ++i) k += poisson_inversion(sub, st.uniform(), rcp);
-    return k;
+    // at most four further uniforms: the first block of the own stream
+    const uint4 b = philox4x32_10(make_uint4((uint32_t)index, (uint32_t)(index >> 32), 1u, tag),
+                                  (uint32_t)seed, (uint32_t)(seed >> 32));
+    const float u[5] = {u0, word_uniform(b.x), word_uniform(b.y), word_uniform(b.z),
+                        word_uniform(b.w)};
+    return poisson_inversions(sub, u, (int)parts);
   }
+  BinStream st(index, seed, tag);
   return poisson_ptrs(lam, st);
 }
 
 // The count of bin `index` given its first uniform u0 (from its group block).
 __device__ __forceinline__ uint32_t poisson_from(float lam, float u0, uint64_t index,
-                                                 uint64_t seed, uint32_t tag, const float* rcp) {
+                                                 uint64_t seed, uint32_t tag) {
   if (!(lam > 0.0f)) return 0u;
-  if (lam < kInvMax) return poisson_inversion(lam, u0, rcp);
-  return poisson_large(lam, u0, index, seed, tag, rcp);
+  if (lam < kInvMax) return poisson_inversion(lam, u0);
+  return poisson_large(lam, u0, index, seed, tag);
 }
 
 // One bin on its own (its group block is computed for it alone).
 __device__ __forceinline__ uint32_t poisson_sample(float lam, uint64_t index, uint64_t seed,
-                                                   uint32_t tag, const float* rcp = nullptr) {
+                                                   uint32_t tag) {
   if (!(lam > 0.0f)) return 0u;
   const uint4 b = group_block(index >> 2, seed, tag);
-  return poisson_from(lam, word_uniform(group_word(b, (uint32_t)(index & 3u))), index, seed, tag,
-                      rcp);
-}
-
-// Fills a shared table of 1/k (k < kRcpTable; entry 0 unused) with nthreads
-// threads starting at thread t0; the caller synchronises before use.
-__device__ __forceinline__ void fill_rcp_table(float* rcp, int t, int nthreads) {
-  for (int k = t; k < kRcpTable; k += nthreads) rcp[k] = k ? __frcp_rn((float)k) : 0.0f;
+  return poisson_from(lam, word_uniform(group_word(b, (uint32_t)(index & 3u))), index, seed, tag);
 }
 
 // Counts of the bins [b, e) of a cube part (local indices; the global index
@@ -186,7 +233,7 @@ template <bool DEFER = false>
 __device__ __forceinline__ void noise_groups(const float* __restrict__ tau,
                                              uint32_t* __restrict__ counts, uint64_t b, uint64_t e,
                                              uint64_t index_base, float scale, float dark,
-                                             uint64_t seed, uint32_t tag, const float* rcp,
+                                             uint64_t seed, uint32_t tag,
                                              uint64_t j0, uint64_t stride,
                                              const DeferList* dl = nullptr) {
   if (b >= e) return;
@@ -218,10 +265,10 @@ __device__ __forceinline__ void noise_groups(const float* __restrict__ tau,
       const float u0 = word_uniform(group_word(blk, (uint32_t)r));
       if (DEFER)
         c[r] = !(lam > 0.0f) ? 0u
-               : lam < kInvMax ? poisson_inversion(lam, u0, rcp)
+               : lam < kInvMax ? poisson_inversion(lam, u0)
                                : kDeferredCount;
       else
-        c[r] = poisson_from(lam, u0, 4 * g + r, seed, tag, rcp);
+        c[r] = poisson_from(lam, u0, 4 * g + r, seed, tag);
     }
     if (DEFER) {
       uint32_t dm = 0;  // bit r: bin 4g + r was deferred
@@ -273,12 +320,11 @@ __device__ __forceinline__ void noise_groups(const float* __restrict__ tau,
 __device__ __forceinline__ void noise_deferred_bin(const float* __restrict__ tau,
                                                    uint32_t* __restrict__ counts, uint64_t l,
                                                    uint64_t index_base, float scale, float dark,
-                                                   uint64_t seed, uint32_t tag, const float* rcp) {
+                                                   uint64_t seed, uint32_t tag) {
   const uint64_t i = index_base + l;
   const float lam = fmaf(scale, __ldg(tau + l), dark);
   const uint4 blk = group_block(i >> 2, seed, tag);
-  counts[l] = poisson_large(lam, word_uniform(group_word(blk, (uint32_t)(i & 3u))), i, seed, tag,
-                            rcp);
+  counts[l] = poisson_large(lam, word_uniform(group_word(blk, (uint32_t)(i & 3u))), i, seed, tag);
 }
 
 // Second pass over one 32-group region (global bins 4 G0 .. 4 G0 + 127; local
@@ -290,7 +336,7 @@ __device__ __forceinline__ void noise_deferred_warp(const float* __restrict__ ta
                                                     uint32_t* __restrict__ counts, uint64_t n,
                                                     uint64_t G0, uint64_t index_base,
                                                     float scale, float dark, uint64_t seed,
-                                                    uint32_t tag, const float* rcp) {
+                                                    uint32_t tag) {
   const uint32_t lane = threadIdx.x & 31u;
   const int64_t w0 = (int64_t)(4 * G0) - (int64_t)index_base;
   uint32_t m[4];
@@ -314,7 +360,7 @@ __device__ __forceinline__ void noise_deferred_warp(const float* __restrict__ ta
       for (uint32_t j = 0; j < k; ++j) mm &= mm - 1u;  // drop the k lowest set bits
       const uint32_t src = (uint32_t)__ffs((int)mm) - 1u;
       const int64_t l = w0 + 32 * r + (int64_t)src;
-      noise_deferred_bin(tau, counts, (uint64_t)l, index_base, scale, dark, seed, tag, rcp);
+      noise_deferred_bin(tau, counts, (uint64_t)l, index_base, scale, dark, seed, tag);
     }
   }
 }

@@ -275,7 +275,7 @@ __device__ __noinline__ void noise_item(const JobDesc& j, uint64_t b, uint64_t e
   }
   // groups of four bins (one Philox block for their first draws); a group
   // that straddles an item edge is drawn by both items, each keeping its bins
-  noise_groups(j.fwd.tau, j.counts, b, e, 0, scale, j.dark, j.seed, j.tag, nullptr, threadIdx.x,
+  noise_groups(j.fwd.tau, j.counts, b, e, 0, scale, j.dark, j.seed, j.tag, threadIdx.x,
                blockDim.x);
 }
 
