@@ -106,7 +106,8 @@ __device__ __forceinline__ void leg_length(float r2, float& r, float& ri) {
 // summation, and a rounded sum of the legs where the compiler would fuse it.
 template <bool TAPS>
 __device__ __forceinline__ float leg_r2(float vx, float vy, float vz) {
-  return TAPS ? vx * vx + vy * vy + vz * vz : fmaf(vx, vx, fmaf(vy, vy, vz * vz));
+  return TAPS ? __fadd_rn(fmaf(vx, vx, __fmul_rn(vy, vy)), __fmul_rn(vz, vz))
+              : fmaf(vx, vx, fmaf(vy, vy, vz * vz));
 }
 
 // Leg factor F = cosf * wallf / r^2 and its delta-derivative (FP32); ri = 1 / r.
