@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(1024, 1)
   sm.lane_units = sm.units + a.stages + 1;
   sm.rows = reinterpret_cast<uint32_t*>(sm.lane_units + 32);
   sm.fill = sm.rows + kRowWords;
+  sm.occ = sm.fill + kMaxRangedStages;
   if (threadIdx.x == 0) {
     for (uint32_t i = 0; i < a.stages; ++i) {
       mbar_init(&sm.bars[i], 1);                                 // full
@@ -409,7 +410,7 @@ cudaError_t forward_plan_create(SceneImpl& sc) {
   // staged blocks, then full + empty barriers and what each slot holds
   auto stage_bytes = [&]() {
     return a.stages * (size_t)a.ppb * sizeof(PointPair) + 24 * a.stages + 64 + 8 * 32 +
-           4 * kRowWords + 4 * kMaxRangedStages;
+           4 * kRowWords + 4 * kMaxRangedStages + 4 * a.stages * kOccGroups;
   };
   if (moments) {
     // windows of at most kMomRows rows over the bins and J beyond each end
@@ -418,7 +419,9 @@ cudaError_t forward_plan_create(SceneImpl& sc) {
     a.n_win = (bins + max_bw - 1) / max_bw;
     a.bw = (bins + a.n_win - 1) / a.n_win;
   } else {
-    const uint32_t max_bw = (uint32_t)(((size_t)optin - stage_bytes()) / (kTile * 4)) & ~3u;
+    // (256 bytes for the kernel's static shared memory)
+    const uint32_t max_bw =
+        (uint32_t)(((size_t)optin - 256 - stage_bytes()) / (kTile * 4)) & ~3u;
     a.n_win = (g.B + max_bw - 1) / max_bw;
     a.bw = ((g.B + a.n_win - 1) / a.n_win + 3) & ~3u;
   }

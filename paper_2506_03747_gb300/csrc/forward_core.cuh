@@ -357,11 +357,14 @@ struct FwdSmem {
   unsigned long long* units;   // [stages]: the (tile, window) of each slot's pairs
   uint32_t* rows = nullptr;    // [kRowWords] or null: row tracking (see fwd_run_ws)
   uint32_t* fill = nullptr;    // [stages]: the pairs staged in each slot
+  uint32_t* occ = nullptr;     // [stages][kOccGroups]: occluders of each group (MODE_NEAREST_OCC)
   unsigned long long* lane_units = nullptr;  // [32]: the producer lanes' units (list mode)
 };
 // rows: 32 words for the producer's lanes, then one per slot (up to 8 stages)
 constexpr int kMaxRangedStages = 8;
 constexpr int kRowWords = 32 + kMaxRangedStages;
+
+constexpr uint32_t kOccGroups = NLOS_FWD_PPB / kGroupPairs;  // groups of a slot
 
 constexpr unsigned long long kNoUnit = ~0ull;  // end of a run (in FwdSmem::units)
 
@@ -569,7 +572,7 @@ __device__ __forceinline__ void red_moments(uint32_t addr, float w, float c, uin
 // slab intervals of t, with reciprocal estimates. The threshold is far above
 // the FP32 rounding of the chord except for near-tangent segments, which the
 // parity tests treat like pairs near a bin edge. Only the occluders of `mask`
-// (those the unit's segments can meet, occ_unit_mask) are tested.
+// (those the segments to the point's group can meet, occ_bounds_mask) are tested.
 __device__ __forceinline__ bool occ_seen(const OccSet& o, uint32_t mask, float sx, float sy,
                                          float dx, float dy, float dz, float A) {
   for (; mask; mask &= mask - 1) {
@@ -621,7 +624,8 @@ __device__ __forceinline__ void compute_block(const FwdArgs& a, const PointPair*
                                               int warp_rel, int n_warps, const TileState& ts,
                                               uint32_t col_addr, FwdCount& cnt,
                                               int mom_q = 1, const OccSet* occ = nullptr,
-                                              uint32_t occ_mask = 0, uint32_t rot = 0) {
+                                              const uint32_t* occ_groups = nullptr,
+                                              uint32_t rot = 0) {
   const float2 kbin2 = make_float2(a.kbin, a.kbin);
   const float2 magic2 = make_float2(kMagic, kMagic);
   const float2 ikbin_neg = make_float2(-1.0f / a.kbin, -1.0f / a.kbin);
@@ -683,6 +687,7 @@ __device__ __forceinline__ void compute_block(const FwdArgs& a, const PointPair*
         // visibility only for pairs that would be binned; a hidden pair's bin
         // is moved out of range, so its reduction is predicated off
         const float sx = ts.sx2.x, sy = ts.sy2.x;
+        const uint32_t occ_mask = occ_groups[i / kGroupPairs];
         if (ba < (uint32_t)ts.lim && facing<COS>(cn.x) &&
             !occ_seen(*occ, occ_mask, sx, sy, q.px.x - sx, q.py.x - sy, sqrt_approx(q.pz2.x),
                       r2.x))
@@ -925,21 +930,15 @@ __device__ __forceinline__ uint32_t unit_groups(const FwdArgs& a, unsigned long 
   return __ballot_sync(0xffffffffu, live);
 }
 
-// Occluders that can meet a segment from a spot of the unit's tile (z = 0)
-// to a point of its block, as bits (conservative). A segment ending at depth
+// Occluders that can meet a segment from a spot of the tile t (z = 0) to a
+// point inside the bounds b, as bits (conservative). A segment ending at depth
 // z_p in [z0, z1] is at depth zeta at t = zeta / z_p, over the lateral box
 // interpolated at t between the tile's spot box and the block's box; over
 // the depths an occluder spans, t stays in [zeta_lo / z1, min(1, zeta_hi /
 // z0)], and the box is linear in t, so its extremes sit at those two ends.
-// Without bounds every occluder counts.
-__device__ __forceinline__ uint32_t occ_unit_mask(const FwdArgs& a, unsigned long long unit,
-                                                  const OccSet& o) {
+__device__ __forceinline__ uint32_t occ_bounds_mask(const TileBound& t, const BlockBound& b,
+                                                    const OccSet& o) {
   const uint32_t all = o.n >= 32 ? 0xFFFFFFFFu : (1u << o.n) - 1u;
-  if (a.bounds == nullptr) return all;
-  const unsigned long long tw = unit / a.n_blk;
-  const uint32_t blk = (uint32_t)(unit - tw * a.n_blk);
-  const TileBound t = a.tiles[(uint32_t)(tw / a.n_win)];
-  const BlockBound b = block_bound(a, blk);
   if (!(b.z0 > 0.f)) return all;
   constexpr float pad = 1e-4f;  // metres, against rounding of the boxes
   uint32_t m = 0;
@@ -971,10 +970,6 @@ __device__ __forceinline__ uint32_t unit_rows(float ulo, float uhi, float margin
   const float hi = fminf(ceilf(fminf(uhi, 1e6f)) + m + 1.f, (float)bw);
   return lo < hi ? (uint32_t)lo | ((uint32_t)hi << 16) : 0u;
 }
-
-// Units carry the occluder mask of MODE_NEAREST_OCC in their top bits.
-constexpr int kUnitBits = 48;
-constexpr unsigned long long kUnitMask = (1ull << kUnitBits) - 1ull;
 
 __device__ __forceinline__ void named_barrier(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -1099,12 +1094,12 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
     uint32_t run_rows = 0;   // union of the rows of its units so far
     unsigned long long slot_tw = kNoUnit; // of the open slot
     uint32_t fill = 0;       // pairs in the open slot (0: none is open)
-    uint32_t unit_occ = 0, slot_occ = 0;  // occluder masks of the unit and of the open slot
     // hands the open slot to the consumers
     auto commit = [&]() {
+      if (MODE == MODE_NEAREST_OCC) __syncwarp();  // (every lane wrote its groups' masks)
       if (lane == 0) {
         const int slot = (int)((it + k) % (uint32_t)stages);
-        unit_of[slot] = slot_tw | ((unsigned long long)slot_occ << kUnitBits);
+        unit_of[slot] = slot_tw;
         sm.fill[slot] = fill;
         if (ranged) s_slot_rows[slot] = run_rows;
         mbar_arrive(&full[slot]);
@@ -1151,7 +1146,12 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
         if (groups == 0u) continue;
         const unsigned long long utw = unit / a.n_blk;
         if (fill > 0 && utw != slot_tw) commit();
-        if (MODE == MODE_NEAREST_OCC) unit_occ = occ_unit_mask(a, unit, *occ);
+        // each lane's group
+        uint32_t group_occ = 0;
+        if (MODE == MODE_NEAREST_OCC && ((groups >> lane) & 1u))
+          group_occ = occ_bounds_mask(
+              a.tiles[(uint32_t)(utw / a.n_win)],
+              a.groups[((uint32_t)(unit - utw * a.n_blk) * a.ppb) / kGroupPairs + (uint32_t)lane], *occ);
         if (ranged) {
           const uint32_t ur = s_lane_rows[j];
           if (utw != run_tw) {
@@ -1176,9 +1176,7 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
             failed = __shfl_sync(0xffffffffu, (int)failed, 0) != 0;
             if (failed) break;
             slot_tw = utw;
-            slot_occ = 0;
           }
-          slot_occ |= unit_occ;
           // the lowest groups that fit; only the last group of all is short
           const uint32_t room = a.ppb / kGroupPairs - fill / kGroupPairs;
           const uint32_t rank = (uint32_t)__popc(groups & ((1u << lane) - 1u));
@@ -1192,6 +1190,8 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
           __syncwarp();
           if (take) {
             const uint32_t p0 = first + (uint32_t)lane * kGroupPairs;
+            if (MODE == MODE_NEAREST_OCC)
+              sm.occ[slot * kOccGroups + fill / kGroupPairs + rank] = group_occ;
             fence_proxy_async_smem();
             bulk_g2s(sm.stage + (size_t)slot * a.ppb + fill + rank * kGroupPairs, a.pairs + p0,
                      min(kGroupPairs, a.n_pairs - p0) * (uint32_t)sizeof(PointPair), &full[slot]);
@@ -1248,7 +1248,7 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
       }
       const unsigned long long tag = *(volatile unsigned long long*)&unit_of[slot];
       if (tag != kNoUnit) {
-        const long long tw = (long long)(tag & kUnitMask);
+        const long long tw = (long long)tag;
         if (tw != ts.tw) {
           named_barrier(1, nthr);  // every consumer is done with the previous tile
           if (ts.tw >= 0) {
@@ -1274,7 +1274,7 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
         compute_block<SCAN, COS, MODE, UNROLL>(a, sm.stage + (size_t)slot * a.ppb,
                                                *(volatile uint32_t*)&sm.fill[slot], cw, ncw, ts,
                                                col_addr, cnt, mom_q, occ,
-                                               (uint32_t)(tag >> kUnitBits), g);
+                                               sm.occ + slot * kOccGroups, g);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[slot]);
