@@ -241,7 +241,7 @@ nlos_status nlos_scene_shape(const nlos_scene* scene, uint64_t* num_scan, uint32
  *              fills it.
  * Asynchronous on cuda_stream otherwise. Calls on one scene must not overlap
  * on the device (they share its scratch): use one stream per scene.
- * Device memory: the forward's live-unit list (8 bytes a (tile, window, point
+ * Device memory: the forward's live-unit list (16 bytes a (tile, window, point
  * block) unit) and the noise step's deferred-bin lists (about 3% of the bins;
  * noise_mode != NONE) belong to the scene from its creation, whose calls
  * allocate nothing. */

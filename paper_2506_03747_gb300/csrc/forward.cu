@@ -68,49 +68,99 @@ __device__ __forceinline__ void zero_floats(float* p, size_t n) {
   for (size_t i = n / 4 * 4 + t; i < n; i += nt) p[i] = 0.f;
 }
 
-// The live units of a pass, for the forward's chunk claims: one CTA per
-// (tile, window) tests the point blocks against the bounds (unit_live, as
-// the producer warp would) and appends the live ones, with the histogram rows
-// they can touch, to the list (unit | rows << 32). Entries of one (tile,
-// window) are contiguous, so a chunk of the list rarely spans two tiles; the
-// order of the (tile, window) runs in the list does not matter. The same launch
-// zeroes the output that the forward adds to.
+constexpr uint32_t kRunWeight = 10;  // a tile change in groups of work (3 to 14 thousand cycles)
+constexpr int kListThreads = 1024;  // (of fewer blocks than 128 a tile: 256)
+
+// The live units of a pass, for the forward's ranges and chunk claims: one CTA
+// per (tile, window) tests the point blocks against the bounds (unit_live),
+// then the groups of the live ones (the warps take them in turn: the live blocks
+// of a tile are neighbours, mostly of one warp), and appends the
+// units that have any with the histogram rows they can touch. Entries of one
+// (tile, window) are contiguous (a CTA's blocks at a time), so a range of the list
+// rarely spans many tiles; the order of the runs does not matter. Each entry
+// holds the weight of the list before it (both come from one atomic, so they
+// ascend together). The same launch zeroes the output that the forward adds to.
 template <int SCAN, int COS, int MODE>
-__global__ void __launch_bounds__(256) unit_list_kernel(const __grid_constant__ FwdArgs a,
-                                                        unsigned long long* __restrict__ list,
-                                                        unsigned long long* __restrict__ n_live) {
-  __shared__ uint32_t s_warp[8];
+__global__ void __launch_bounds__(kListThreads)
+    unit_list_kernel(const __grid_constant__ FwdArgs a, ListEntry* __restrict__ list,
+                     unsigned long long* __restrict__ n_live) {
+  __shared__ uint32_t s_units[32], s_groups[32], s_n;
+  __shared__ uint32_t s_blk[kListThreads], s_rows[kListThreads], s_mask[kListThreads];
   __shared__ unsigned long long s_base;
   zero_floats(a.tau, (size_t)a.S * a.B);
   if (MODE == MODE_SPLAT_MOM) zero_floats(a.far_mass, a.S);
   const unsigned long long tw = blockIdx.x;
   const float margin = window_margin<MODE>(a);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const TileBound tile = a.tiles[(uint32_t)(tw / a.n_win)];
+  const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
+  const float lim = (float)window_bins(a, w0);
   for (uint32_t b0 = 0; b0 < a.n_blk; b0 += blockDim.x) {
     const uint32_t blk = b0 + threadIdx.x;
     const unsigned long long unit = tw * a.n_blk + blk;
     float ulo = 0.f, uhi = 0.f;
-    const bool live =
+    const bool maybe =
         blk < a.n_blk && (a.ppb == 2 * kSubPairs
                               ? unit_live_halves<SCAN, COS>(a, unit, margin, ulo, uhi)
                               : unit_live<SCAN, COS>(a, unit, margin, ulo, uhi));
-    const uint32_t rows = live ? unit_rows(ulo, uhi, margin, a.bw) : 0u;
-    const uint32_t m = __ballot_sync(0xffffffffu, live);
-    if (lane == 0) s_warp[warp] = __popc(m);
+    const uint32_t found = __ballot_sync(0xffffffffu, maybe);
+    if (lane == 0) s_units[warp] = (uint32_t)__popc(found);
     __syncthreads();
     if (threadIdx.x == 0) {
-      uint32_t tot = 0;
+      uint32_t sum = 0;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        const uint32_t c = s_warp[w];
-        s_warp[w] = tot;
-        tot += c;
+        const uint32_t c = s_units[w];
+        s_units[w] = sum;
+        sum += c;
       }
-      s_base = tot ? atomicAdd(n_live, (unsigned long long)tot) : 0ull;
+      s_n = sum;
     }
     __syncthreads();
-    if (live) {
-      const uint32_t pos = s_warp[warp] + __popc(m & ((1u << lane) - 1u));
-      list[s_base + pos] = unit | ((unsigned long long)rows << 32);
+    if (maybe) {
+      const uint32_t at = s_units[warp] + __popc(found & ((1u << lane) - 1u));
+      s_blk[at] = blk;
+      s_rows[at] = unit_rows(ulo, uhi, margin, a.bw);
+    }
+    __syncthreads();
+    const uint32_t n = s_n;
+    for (uint32_t i = warp; i < n; i += blockDim.x >> 5) {
+      const uint32_t g = block_groups<SCAN, COS>(a, tile, s_blk[i], w0, lim, margin);
+      if (lane == 0) s_mask[i] = g;
+    }
+    __syncthreads();
+    // thread i takes the i-th of them
+    const uint32_t groups = threadIdx.x < n ? s_mask[threadIdx.x] : 0u;
+    const uint32_t mask = __ballot_sync(0xffffffffu, groups != 0u);
+    uint32_t upto = (uint32_t)__popc(groups);  // inclusive sum over the lanes
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+      if (lane >= o) upto += v;
+    }
+    if (lane == 31) {
+      s_units[warp] = (uint32_t)__popc(mask);
+      s_groups[warp] = upto;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t units = 0, sum = 0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        const uint32_t u = s_units[w], g = s_groups[w];
+        s_units[w] = units;
+        s_groups[w] = sum;
+        units += u;
+        sum += g;
+      }
+      // (a run's weight is more than any weight within it, so entries ascend)
+      const unsigned long long weight = ((sum + kRunWeight) >> a.list_shift) + 1u;
+      s_base = units ? atomicAdd(n_live, units | (weight << 32)) : 0ull;
+    }
+    __syncthreads();
+    if (groups != 0u) {
+      const uint32_t pos = (uint32_t)s_base + s_units[warp] + __popc(mask & ((1u << lane) - 1u));
+      const uint32_t before = (uint32_t)(s_base >> 32) +
+                              ((s_groups[warp] + upto - (uint32_t)__popc(groups)) >> a.list_shift);
+      list[pos] = ListEntry{(uint32_t)(tw * a.n_blk + s_blk[threadIdx.x]), s_rows[threadIdx.x],
+                            groups, before};
     }
     __syncthreads();
   }
@@ -212,7 +262,7 @@ TailFn pick_tail(int scan, int cos) {
   if (cos == NLOS_COS_OBJECT) return splat_tail_kernel<NLOS_NONCONFOCAL, NLOS_COS_OBJECT>;
   return splat_tail_kernel<NLOS_NONCONFOCAL, NLOS_COS_OBJECT_WALL>;
 }
-using ListFn = void (*)(FwdArgs, unsigned long long*, unsigned long long*);
+using ListFn = void (*)(FwdArgs, ListEntry*, unsigned long long*);
 
 template <int SCAN, int COS>
 ListFn pick_list_mode(int mode) {
@@ -298,7 +348,7 @@ struct FwdPlan {
   ListFn list_fn = nullptr;  // null: chunks of all units are claimed
   size_t smem = 0;
   unsigned grid = 0;
-  unsigned long long* list = nullptr;  // [units], or null
+  ListEntry* list = nullptr;  // [units], or null
 };
 
 namespace {
@@ -447,13 +497,14 @@ cudaError_t forward_plan_create(SceneImpl& sc) {
   // units of which most may be culled, so tile changes (flush, zeroing,
   // barriers) are fewer per unit of work. Without memory for it the producers
   // test the units themselves.
-  if (NLOS_FWD_CULL && mode != MODE_NEAREST_COUNT &&
-      cudaMalloc(reinterpret_cast<void**>(&p->list), sizeof(unsigned long long) * a.units) !=
+  if (NLOS_FWD_CULL && mode != MODE_NEAREST_COUNT && a.units < (1ull << 32) &&
+      cudaMalloc(reinterpret_cast<void**>(&p->list), sizeof(ListEntry) * a.units) !=
           cudaSuccess) {
     p->list = nullptr;
     (void)cudaGetLastError();
   }
   a.unit_list = p->list;
+  while (((a.units * (a.ppb / kGroupPairs)) >> a.list_shift) >= (1ull << 31)) ++a.list_shift;
   a.n_live = &sc.scratch->n_live;
   a.list_chunks_per_cta = NLOS_FWD_LIST_CHUNKS_PER_CTA;
   a.list_min_chunk = NLOS_FWD_LIST_MIN;
@@ -481,7 +532,8 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
   a.tau = tau;
   if (p->list_fn) {
     // (the counters, n_live among them, were zeroed with the pass's scratch)
-    p->list_fn<<<(unsigned)(a.units / a.n_blk), 256, 0, st>>>(a, p->list, &sc.scratch->n_live);
+    p->list_fn<<<(unsigned)(a.units / a.n_blk), a.n_blk < 128 ? 256 : kListThreads, 0, st>>>(
+        a, p->list, &sc.scratch->n_live);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   p->fn<<<p->grid, 1024, p->smem, st>>>(a, p->mt, sc.occ);

@@ -134,6 +134,12 @@ struct FwdCount {
   unsigned long long tested = 0;    // warp iterations of staged units (x 64 pairs)
 };
 
+// A live unit: its number, the histogram rows it can touch (unit_rows), its live
+// groups (unit_groups), and the weight of the list before it.
+struct __align__(16) ListEntry {
+  uint32_t unit, rows, groups, before;
+};
+
 struct FwdArgs {
   const PointPair* pairs;
   const ScanPoint* scan;
@@ -148,14 +154,15 @@ struct FwdArgs {
   unsigned long long* next_chunk;  // standalone launch: chunk counter (zeroed per pass)
   unsigned long long units;   // standalone launch: total units
   unsigned long long chunk;   // standalone launch: units per claimed chunk
-  // standalone launch with a unit list (unit_list_kernel): the live units, as
-  // unit | rows << 32 (rows: unit_rows), *n_live of them; chunks of the list
-  // are claimed instead of chunks of units (null: no list)
-  const unsigned long long* unit_list;
+  // standalone launch with a unit list (unit_list_kernel): *n_live packs its
+  // entries (low word) and their weight (high word: live groups >> list_shift);
+  // chunks of the list are claimed instead of chunks of units (null: no list)
+  const ListEntry* unit_list;
   const unsigned long long* n_live;
+  uint32_t list_shift;
   uint32_t list_chunks_per_cta;  // list chunks per CTA (mean), of the claimed part
   uint32_t list_min_chunk, list_max_chunk;  // list entries per chunk, clamped
-  uint32_t list_static_pct;  // the list's first part (percent) in one contiguous range per CTA
+  uint32_t list_static_pct;  // the list's first part (percent of weight) in one range per CTA
   uint32_t n_pairs, S, B, bw, n_win, n_blk, ppb;
   int halo;          // bins the windows reach beyond [0, B) on each side (moment form: J)
   uint32_t stages;   // staged point blocks (standalone warp-specialised kernel)
@@ -358,7 +365,7 @@ struct FwdSmem {
   uint32_t* rows = nullptr;    // [kRowWords] or null: row tracking (see fwd_run_ws)
   uint32_t* fill = nullptr;    // [stages]: the pairs staged in each slot
   uint32_t* occ = nullptr;     // [stages][kOccGroups]: occluders of each group (MODE_NEAREST_OCC)
-  unsigned long long* lane_units = nullptr;  // [32]: the producer lanes' units (list mode)
+  unsigned long long* lane_units = nullptr;  // [32]: the producer lanes' units | groups << 32 (list)
 };
 // rows: 32 words for the producer's lanes, then one per slot (up to 8 stages)
 constexpr int kMaxRangedStages = 8;
@@ -811,6 +818,31 @@ __device__ __forceinline__ void flush_tile_mom(const FwdArgs& a, const MomTab& m
   if (s < a.S && far != 0.f) red_add_global(a.far_mass + s, far);
 }
 
+// For three weights x at a time, the first of n list entries with at least x
+// before it (n if none), by a whole warp: 32 probes a round.
+__device__ __forceinline__ void list_lower_bounds(const ListEntry* list, uint32_t n,
+                                                  const uint32_t x[3], uint32_t at[3]) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t lo[3] = {0u, 0u, 0u}, len[3] = {n, n, n};
+  while (len[0] | len[1] | len[2]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const uint32_t step = (len[i] + 31u) / 32u, p = lane * step;
+      const bool below = p < len[i] && list[lo[i] + p].before < x[i];
+      const uint32_t m = __ballot_sync(0xffffffffu, below);
+      // probes ascend: the answer lies in (last below, next probe]
+      if (m == 0u) {
+        len[i] = 0u;
+      } else {
+        const uint32_t last = (31u - (uint32_t)__clz((int)m)) * step;
+        lo[i] += last + 1u;
+        len[i] = min(step - 1u, len[i] - last - 1u);
+      }
+    }
+  }
+  for (int i = 0; i < 3; ++i) at[i] = lo[i];
+}
+
 // max of a * b over a in [a0, a1], b in [b0, b1]
 __device__ __forceinline__ float imax(float a0, float a1, float b0, float b1) {
   return fmaxf(fmaxf(a0 * b0, a0 * b1), fmaxf(a1 * b0, a1 * b1));
@@ -909,25 +941,34 @@ __device__ __forceinline__ bool unit_live_halves(const FwdArgs& a, unsigned long
   return live0 || live1;
 }
 
-// The groups of kGroupPairs pairs of a unit that its tile may bin (bit g: pairs
+// The groups of kGroupPairs pairs of a block that a tile may bin (bit g: pairs
 // [16 g, 16 g + 16) of the block), one group a lane; the whole warp calls it.
-// cull: whether to test the groups' bounds (else every group of the block).
+template <int SCAN, int COS>
+__device__ __forceinline__ uint32_t block_groups(const FwdArgs& a, const TileBound& t, uint32_t blk,
+                                                 int w0, float lim, float margin) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t first = blk * a.ppb + lane * kGroupPairs;
+  bool live = lane * kGroupPairs < a.ppb && first < a.n_pairs;
+  if (live) {
+    float ulo, uhi;
+    live = bounds_live<SCAN, COS>(a, t, a.groups[first / kGroupPairs], w0, lim, margin, ulo, uhi);
+  }
+  return __ballot_sync(0xffffffffu, live);
+}
+
+// The same for a unit; cull: whether to test the bounds (else every group).
 template <int SCAN, int COS>
 __device__ __forceinline__ uint32_t unit_groups(const FwdArgs& a, unsigned long long unit,
                                                 float margin, bool cull) {
-  const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long tw = unit / a.n_blk;
   const uint32_t blk = (uint32_t)(unit - tw * a.n_blk);
-  const uint32_t first = blk * a.ppb + lane * kGroupPairs;
-  bool live = lane * kGroupPairs < a.ppb && first < a.n_pairs;
-  if (live && cull) {
-    const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
-    float ulo, uhi;
-    live = bounds_live<SCAN, COS>(a, a.tiles[(uint32_t)(tw / a.n_win)],
-                                  a.groups[first / kGroupPairs], w0,
-                                  (float)window_bins(a, w0), margin, ulo, uhi);
+  if (!cull) {
+    const uint32_t at = (threadIdx.x & 31u) * kGroupPairs;
+    return __ballot_sync(0xffffffffu, at < a.ppb && blk * a.ppb + at < a.n_pairs);
   }
-  return __ballot_sync(0xffffffffu, live);
+  const int w0 = window_start(a, (uint32_t)(tw % a.n_win));
+  return block_groups<SCAN, COS>(a, a.tiles[(uint32_t)(tw / a.n_win)], blk, w0,
+                                 (float)window_bins(a, w0), margin);
 }
 
 // Occluders that can meet a segment from a spot of the tile t (z = 0) to a
@@ -981,9 +1022,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 
 // Warp-specialised run of work units (tile, window, point block) of one job:
 // warp 0 stages points with TMA bulk copies into `stages` slots, the other warps
-// evaluate them. The producer tests the bounds of each group of 16 pairs of a
-// unit, one group a lane, and copies the groups that the tile may bin side by
-// side, so a slot holds up to ppb pairs of one (tile, window), of as many units
+// evaluate them. The bounds of each group of 16 pairs of a unit are tested, one
+// group a lane (by the list's kernel, or here without a list), and the producer
+// copies the groups that the tile may bin side by side, so a slot holds up to ppb pairs of one (tile, window), of as many units
 // as it takes, and the consumers split them evenly. (Evaluating whole blocks,
 // or halves of them, took 24% more pairs on the 64 x 64 union scene and 35%
 // more on a ragged heightfield; skipping dead groups on the consumers' side
@@ -1039,16 +1080,32 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
     // list mode: chunks of the live-unit list, sized from its length
     const bool listed = a.unit_list != nullptr && chunk_counter != nullptr &&
                         sm.lane_units != nullptr;
-    // the list's first list_static_pct percent goes to the CTAs in equal
-    // contiguous ranges (the list holds each (tile, window)'s units together,
-    // so a CTA meets few tiles there); the rest is claimed chunk by chunk
-    // (the claimed part's first entry is kept in shared memory: it is read
-    // once per claim, and a register for it spilled in the pair loop)
+    // the list's first list_static_pct percent (by weight, so that every CTA
+    // gets as many live groups) goes to the CTAs in contiguous ranges (the
+    // list holds each (tile, window)'s units together, so a CTA meets few tiles
+    // there); the rest is claimed chunk by chunk (the claimed part's first entry
+    // is kept in shared memory: it is read once per claim, and a register for it
+    // spilled in the pair loop)
+    unsigned long long s0 = 0, s1 = 0;  // the CTA's range
     if (lane == 0) s_list_base = 0;
     __syncwarp();
     if (listed) {
-      units_total = *reinterpret_cast<const volatile unsigned long long*>(a.n_live);
-      if (lane == 0) s_list_base = units_total * a.list_static_pct / 100ull;
+      const unsigned long long nl = *reinterpret_cast<const volatile unsigned long long*>(a.n_live);
+      units_total = nl & 0xFFFFFFFFull;
+      // chunks of a short list would hold too few units for the flush that
+      // each costs: its whole weight goes out in the ranges (a ragged scan of
+      // 1,500 live units: 66 against 76 us; a heightfield of 50,000 balances
+      // better with claims, 1,062 against 1,257 us)
+      const bool claimed = units_total * (100u - a.list_static_pct) / 100ull >=
+                           4ull * gridDim.x * a.list_chunks_per_cta;
+      const unsigned long long share = claimed ? (nl >> 32) * a.list_static_pct / 100ull : nl >> 32;
+      const uint32_t x[3] = {(uint32_t)(share * blockIdx.x / gridDim.x),
+                             (uint32_t)(share * (blockIdx.x + 1ull) / gridDim.x), (uint32_t)share};
+      uint32_t at[3];
+      list_lower_bounds(a.unit_list, (uint32_t)units_total, x, at);
+      s0 = at[0];
+      s1 = at[1];
+      if (lane == 0) s_list_base = at[2];
       __syncwarp();
       chunk = (units_total - s_list_base) /
               ((unsigned long long)gridDim.x * a.list_chunks_per_cta);
@@ -1067,8 +1124,8 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
     if (chunk_counter) {
       const unsigned long long base = s_list_base;
       if (base > 0) {
-        cur = base * blockIdx.x / gridDim.x;
-        lim = base * (blockIdx.x + 1ull) / gridDim.x;
+        cur = s0;
+        lim = s1;
       } else {
         const unsigned long long c = claim();
         cur = min(c * chunk, units_total);
@@ -1121,11 +1178,12 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
       const uint32_t n = (uint32_t)min(32ull, lim - cur);
       bool live;
       if (listed) {
-        // every list entry is live; its rows were found with it
+        // every list entry is live; its rows and groups were found with it
         live = lane < n;
-        const unsigned long long e = live ? a.unit_list[cur + lane] : 0ull;
-        sm.lane_units[lane] = e & 0xFFFFFFFFull;
-        if (ranged) s_lane_rows[lane] = (uint32_t)(e >> 32);
+        uint4 e = make_uint4(0u, 0u, 0u, 0u);
+        if (live) e = reinterpret_cast<const uint4*>(a.unit_list)[cur + lane];
+        sm.lane_units[lane] = e.x | ((unsigned long long)e.z << 32);
+        if (ranged) s_lane_rows[lane] = e.y;
         __syncwarp();
       } else {
         float ulo = 0.f, uhi = 0.f;
@@ -1141,8 +1199,9 @@ __device__ bool fwd_run_ws(const FwdArgs& a, unsigned long long u0, unsigned lon
       while (mask && !failed) {
         const int j = __ffs(mask) - 1;
         mask &= mask - 1;
-        const unsigned long long unit = listed ? sm.lane_units[j] : cur + j;
-        uint32_t groups = unit_groups<SCAN, COS>(a, unit, margin, cull);
+        const unsigned long long unit = listed ? (sm.lane_units[j] & 0xFFFFFFFFull) : cur + j;
+        uint32_t groups = listed ? (uint32_t)(sm.lane_units[j] >> 32)
+                                 : unit_groups<SCAN, COS>(a, unit, margin, cull);
         if (groups == 0u) continue;
         const unsigned long long utw = unit / a.n_blk;
         if (fill > 0 && utw != slot_tw) commit();
