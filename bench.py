@@ -147,27 +147,22 @@ class ClockSampler:
 
 
 FORWARD_SOURCES = ("forward.cu", "forward_core.cuh", "device_util.cuh", "common.cuh")
-# FP32 issue slots per (scan point, point) pair of the moment-form adjoint
-# kernel, counted from its source: per leg the differences, squared length
-# and square root (2 + 3 + 4), the normal's dot product (3), the reciprocal,
-# cosine, its derivative and the 1/r^2 factor (18), 30 a leg; then the weight
-# and its two derivatives (8), u and du/d(delta) (4), the moment row and c (5),
-# two 6-term Horner evaluations and G1 (12), the two products (4), 33 in all.
-# A pair evaluates one leg: a confocal scan's laser spot is its detector spot,
-# and a non-confocal scan's laser leg depends on the point only (the kernel
-# computes it once per point): 63 (a few of these are integer or select
-# instructions).
-ADJ_FP32_SLOTS_PER_PAIR = {"confocal": 63, "nonconfocal": 63}
+# FP32 issue slots of the moment-form adjoint: of every (scan point, point) pair
+# (differences 2, squared length 3, reciprocal square root step and length 4,
+# path bin 1), and of a pair that reaches the window and faces its spot
+# (cosine 3, weight and its derivative 8, row and offset 5, the two Horner
+# schemes 14, sums 4).
+ADJ_FP32_SLOTS_LEG = 10
+ADJ_FP32_SLOTS_REST = 34
 
 
 def launches_per_step(split: bool) -> int:
-    """Kernels of this library one bench step launches: the ingest (counts and
-    box initialised, bounding box, Morton cells, the scan of the cell counts,
-    the scatter, pack + block bounds), the forward (live-unit list, pair
-    histogram), and the detect step (reduce; noise and its second pass over the
-    deferred bright bins); a split cube reduces through nlos_reduce, which adds
-    the statistics copy kernel."""
-    return 6 + 2 + (4 if split else 3)
+    """Kernels of this library one bench step launches: the ingest (ordering,
+    pack + bounds), the forward (live-unit list, pair histogram), and the
+    detect step (reduce; noise and its second pass over the deferred bright
+    bins); a split cube reduces through nlos_reduce, which adds the statistics
+    copy kernel."""
+    return 2 + 2 + (4 if split else 3)
 
 
 def forward_sources_sha256() -> str:
@@ -283,7 +278,7 @@ def forward_roofline(name, fwd_s, st, pairs_per_step, n_sm, sm_max_mhz, peaks, S
                           f"{MUFU_PER_PAIR} per pair = {mufu_peak / 1e9:.0f} Gpair/s), {basis}",
             "work_basis": f"full-evaluation-equivalent pairs: pairs evaluated in full + "
                           f"{FP32_SLOTS_EARLY_OUT}/{FP32_SLOTS_PER_PAIR} x pairs stopped by "
-                          f"the early out; pairs of units ruled out by the block bounds "
+                          f"the early out; pairs of groups ruled out by their bounds "
                           f"count 0",
             "pairs_full_fraction": full / pairs_per_step,
             "pairs_tested_fraction": tested / pairs_per_step,
@@ -636,21 +631,15 @@ def lct_bench(steps: int, peaks=None):
     return out
 
 
-def splat_moment_reds(params, pts, n_sample=128, seed=7):
-    """Shared reductions per pass of the moment-form splat forward, counted on
-    the host on a sample of scan points and scaled to the scan: six per
-    (pair, bin window) whose moment row floor(u) - w0 + J lies inside the
-    window's bw + 2J rows, for facing pairs of nonzero weight (the kernel's
-    predicate). Windows as the launch chooses them: J = ceil(6 sigma) + 1,
-    at most 256 - 2J bins each, rounded up to multiples of 4."""
+def splat_landed_pairs(params, pts, n_sample=128, seed=7):
+    """Pairs of a confocal splat scene without stand-off that reach the window
+    (bins -J to B + J, J = ceil(6 sigma) + 1) with nonzero weight, facing the
+    spot: those whose moments the forward adds and whose gradient the adjoint
+    evaluates. Counted on the host on a sample of scan points, scaled to the scan."""
     import math
     C = 299792458.0
     sig = params["jitter_fwhm_s"] / (2.0 * math.sqrt(2.0 * math.log(2.0)) * params["bin_width_s"])
     J = math.ceil(6.0 * sig) + 1
-    B = params["num_bins"]
-    max_bw = (256 - 2 * J) & ~3
-    n_win = -(-B // max_bw)
-    bw = ((-(-B // n_win)) + 3) & ~3
     nx, ny, w = params["scan_nx"], params["scan_ny"], params["wall_half_x"]
     rng = np.random.default_rng(seed)
     S = nx * ny
@@ -664,12 +653,10 @@ def splat_moment_reds(params, pts, n_sample=128, seed=7):
     r = np.sqrt(dx * dx + dy * dy + p[None, :, 2] ** 2)
     cn = p[None, :, 3] * dx + p[None, :, 4] * dy - p[None, :, 5] * p[None, :, 2]
     j = np.floor(2.0 * r / (C * params["bin_width_s"]))  # no stand-off, L0 = 0
-    ok = (cn > 0) & (q[None, :] > 0)
-    count = 0
-    for k in range(n_win):
-        row = j - k * bw + J
-        count += int(((row >= 0) & (row < bw + 2 * J) & ok).sum())
-    return 6.0 * count * S / len(ids)
+    inside = (cn > 0) & (j >= -J) & (j < params["num_bins"] + J)
+    # (the adjoint also evaluates pairs of albedo 0)
+    return (float((inside & (q[None, :] > 0)).sum()) * S / len(ids),
+            float(inside.sum()) * S / len(ids))
 
 
 def splat_adjoint_bench(steps: int, warmup: int, peaks=None):
@@ -740,7 +727,8 @@ def splat_adjoint_bench(steps: int, warmup: int, peaks=None):
     if peaks:
         props = torch.cuda.get_device_properties(torch.cuda.current_device())
         f_max = 2070e6
-        reds = sum(splat_moment_reds(params, p) for p in sc_pts)
+        landed = [splat_landed_pairs(params, p) for p in sc_pts]
+        reds = 6.0 * sum(n for n, _ in landed)
         achieved = steps * reds / f
         peak = props.multi_processor_count * peaks["red_f32"] * f_max
         out["forward_roofline"] = {
@@ -748,22 +736,22 @@ def splat_adjoint_bench(steps: int, warmup: int, peaks=None):
             "unit": "G red.shared.add.f32 lanes/s", "frac": achieved / peak,
             "peak_basis": f"{props.multi_processor_count} SMs x {peaks['red_f32']:.2f} lanes/clk "
                           f"(measured, all lanes active) x 2070 MHz",
-            "work_basis": "6 reductions per (pair, bin window) with the moment row in range, "
-                          "counted on the host on 128 sampled scan points per scene"}
-        # FP32 roofline of the adjoint (moment form): every (scan point, point)
-        # pair is evaluated, at ADJ_FP32_SLOTS_PER_PAIR FP32 issue slots each
-        slots = ADJ_FP32_SLOTS_PER_PAIR[params.get("scan_mode", "confocal")]
-        adj_peak = props.multi_processor_count * peaks["ffma"] * f_max / slots
-        adj = steps * pairs / b
+            "work_basis": "6 reductions per pair that reaches the window, counted on the host "
+                          "on 128 sampled scan points per scene"}
+        # FP32 roofline of the adjoint (moment form): the leg of every pair, the
+        # rest of the pairs that reach the window and face the spot
+        work = pairs * ADJ_FP32_SLOTS_LEG + sum(n for _, n in landed) * ADJ_FP32_SLOTS_REST
+        adj_peak = props.multi_processor_count * peaks["ffma"] * f_max
+        adj = steps * work / b
         out["adjoint_roofline"] = {
-            "bound": "alu", "achieved": adj / 1e9, "peak": adj_peak / 1e9, "unit": "Gpair/s",
+            "bound": "alu", "achieved": adj / 1e9, "peak": adj_peak / 1e9, "unit": "G FP32 slots/s",
             "frac": adj / adj_peak,
             "peak_basis": f"{props.multi_processor_count} SMs x {peaks['ffma']:.1f} FMA lanes/clk "
-                          f"(measured) x 2070 MHz / {slots} slots per pair "
-                          f"({params.get('scan_mode', 'confocal')} scan)",
-            "work_basis": "all S x P pairs (the adjoint culls none); its time includes the "
-                          "moment-table kernel; 48 B per pair gathered from the L2-resident "
-                          "moment tables"}
+                          f"(measured) x 2070 MHz",
+            "work_basis": f"{ADJ_FP32_SLOTS_LEG} slots for each of the S x P pairs and "
+                          f"{ADJ_FP32_SLOTS_REST} more for those that reach the window and face "
+                          f"the spot (128 sampled scan points per scene); the time includes the "
+                          f"moment-table kernel"}
     return out
 
 
