@@ -221,7 +221,8 @@ constexpr uint32_t kDeferredCount = 0xFFFFFFFFu;
 // (count in hdr[0], at most cap entries) and, for a warp whose bins no longer
 // fit, the first group of its 32-group region (count in hdr[1]); the lanes of
 // a warp take consecutive groups (j0 = 32 * warp + lane, stride a multiple of
-// 32), so the lanes still in the loop are always a prefix of the warp.
+// 32), so the lanes still in the loop are always a prefix of the warp, whose
+// length follows from the group numbers alone.
 struct DeferList {
   unsigned long long* hdr;       // [2]: dense entries claimed, regions listed
   uint32_t* bins;                // [cap] local bin indices (kDeferredCount: skip)
@@ -274,9 +275,13 @@ __device__ __forceinline__ void noise_groups(const float* __restrict__ tau,
       uint32_t dm = 0;  // bit r: bin 4g + r was deferred
 #pragma unroll
       for (int r = 0; r < 4; ++r) dm |= (uint32_t)(c[r] == kDeferredCount) << r;
-      const uint32_t act = __activemask();
+      // the searches above end in each lane on its own: the lanes of this step
+      // are counted, not taken from those that happen to arrive together
+      const uint32_t lane = threadIdx.x & 31u;
+      const uint64_t in_step = ge - (g - lane);
+      const uint32_t act = in_step >= 32u ? 0xFFFFFFFFu : (1u << (uint32_t)in_step) - 1u;
+      __syncwarp(act);
       if (__any_sync(act, dm != 0u)) {
-        const uint32_t lane = threadIdx.x & 31u;
         const uint32_t cnt = (uint32_t)__popc(dm);
         uint32_t incl = cnt;  // inclusive prefix sum over the lanes (a prefix of the warp)
 #pragma unroll
