@@ -276,10 +276,10 @@ nlos_status nlos_noise_part(nlos_scene* scene, const float* tau_dev, uint32_t* c
  * grad_tau_dev must be 16-byte aligned. Asynchronous on cuda_stream; the
  * outputs are zeroed, then accumulated with global atomics (the order of the
  * FP32 additions, and so the last bits, may differ from call to call).
- * Device memory: for a splat of sigma up to 9.8 bins (the moment form) tables
- * of 32 bytes a row of a transient's B + 2J bins (J = ceil(6 sigma) + 1; one row
- * a bin from sigma = 2.5 up, two to sixteen below), of as many transients at a
- * time as 64 MiB hold and at least one, allocated with cudaMallocAsync and
+ * Device memory: in the moment form (sigma up to 9.8 bins; below 1.5625 bins
+ * only with enough points a bin) tables of 32 bytes a row of a transient's
+ * B + 2J bins (J = ceil(6 sigma) + 1; one row a bin from sigma = 2.5 up, two to
+ * sixteen below), of as many transients at a time as 64 MiB hold and at least one, allocated with cudaMallocAsync and
  * freed on the same stream; NLOS_ECUDA when they cannot be allocated. */
 nlos_status nlos_simulate_backward(nlos_scene* scene, const float* grad_tau_dev,
                                    float* grad_albedo_dev, float* grad_depth_dev,

@@ -9,7 +9,7 @@
 // with, for x -> x + delta n: dr/d delta = -cos, d cos/d delta = -(1 - cos^2)/r,
 // d(z/r)/d delta = (n_z + (z/r) cos)/r and du/d delta = -(cos_l + cos_d)/(c dt).
 //
-// Two forms of the sums G0, G1:
+// Two forms of the sums G0, G1 (adjoint_moments chooses):
 //  * taps (any sigma): one CTA per (32-scan-point tile, point block); the
 //    tile's g rows are staged into shared memory as [bin][32] (lane = scan
 //    point, conflict-free gathers) and each lane runs the |x_b| < 6 sigma taps
@@ -449,8 +449,9 @@ cudaError_t launch_backward(const SceneImpl& sc, const float* grad_tau, float* g
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, sc.device);
   // the taps form holds a transient's bins in shared memory; splats below 2.5
   // bins, which it used to serve, keep its limit on their number
-  if ((s < 2.5 || !use_moments(s)) && smem > (size_t)optin) return cudaErrorInvalidValue;
-  if (use_moments(s)) {
+  const bool moments = adjoint_moments(s, g.P, g.B);
+  if ((s < 2.5 || !moments) && smem > (size_t)optin) return cudaErrorInvalidValue;
+  if (moments) {
     // moment tables of as many transients as kAdjTabBytes hold (in L2, where
     // the pair kernel gathers from them), stream-ordered, freed after use
     MomTab mt;

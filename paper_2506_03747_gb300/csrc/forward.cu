@@ -355,7 +355,8 @@ namespace {
 
 int forward_mode(const SceneImpl& sc) {
   const Geometry& g = sc.g;
-  return g.bin_mode == NLOS_BIN_SPLAT ? (use_moments(g.sigma) ? MODE_SPLAT_MOM : MODE_SPLAT)
+  return g.bin_mode == NLOS_BIN_SPLAT ? (forward_moments(g.sigma, g.P, g.B) ? MODE_SPLAT_MOM
+                                                                                : MODE_SPLAT)
          : sc.params.boundary_eps > 0.f ? MODE_NEAREST_COUNT
          : sc.occ.n > 0                 ? MODE_NEAREST_OCC
                                         : MODE_NEAREST;

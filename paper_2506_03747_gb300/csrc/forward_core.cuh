@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "device_util.cuh"
+#include "rules.h"
 
 #include <cmath>
 
@@ -95,15 +96,14 @@ enum { MODE_NEAREST = 0, MODE_NEAREST_COUNT = 1, MODE_SPLAT = 2, MODE_SPLAT_MOM 
 // that could show, in a transient that holds little but the cut tails of
 // pairs beyond its ends, splat_tail_kernel sums the taps instead. A pair costs six shared reductions at
 // any sigma, against 12 sigma of its taps: a 32 x 32 scan of 16,384 points at
-// sigma = 1.6 takes 0.139 ms against 2.63 ms pair by pair. Fewer moments on
+// sigma = 1.6 takes 0.139 ms against 2.63 ms pair by pair (forward_moments says
+// where the taps remain the better form). Fewer moments on
 // finer rows (five at 0.1 sigma, four at 0.05) reduce less a pair but cut the
 // windows into more: 0.74 and 0.79 ms against 0.68 ms (64 x 64 scan, 65,536
 // points, sigma = 3.2).
 constexpr int kMoments = 6;       // of the forward
 constexpr int kMomTerms = 8;      // terms of the table (the adjoint takes them all)
 constexpr int kMomRows = 256;
-constexpr int kMomMaxJ = 60;
-constexpr int kMomTaps = 144;     // (2J + 1) q at most: 121 at q = 1, 66, 92, 104, 144 at q = 2 .. 16
 constexpr uint32_t kMomStride = kMomRows * 32 * 4;  // bytes between moment histograms
 struct __align__(16) MomTab {
   int J, q;
@@ -112,20 +112,6 @@ struct __align__(16) MomTab {
 
 // Fills mt for the unit-area Gaussian of standard deviation s bins (host).
 void moment_table(double s, MomTab& mt);
-
-// Rows a bin of the moment form.
-inline int moment_rows_per_bin(double sigma) {
-  int q = 1;
-  if (sigma < 2.5)
-    while (0.5 / q > 0.16 * sigma) q *= 2;
-  return q;
-}
-
-// The moment form is used for splat kernels whose taps fit MomTab (sigma up
-// to 9.8 bins); wider ones run their taps pair by pair.
-inline bool use_moments(double sigma) {
-  return (int)std::ceil(6.0 * sigma) + 1 <= kMomMaxJ;
-}
 
 // Per-thread counters of one forward run, added to the scene scratch at exit.
 struct FwdCount {

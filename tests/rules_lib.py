@@ -1,0 +1,32 @@
+"""The library's host rules (csrc/rules.h, plain C++) compiled for the tests."""
+import ctypes
+import os
+import subprocess
+import tempfile
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = """
+#include "rules.h"
+using namespace nlos;
+extern "C" {
+int rows_per_bin(double s) { return moment_rows_per_bin(s); }
+int fits(double s) { return moments_fit(s); }
+int max_j() { return kMomMaxJ; }
+int max_taps() { return kMomTaps; }
+int forward_mom(double s, uint64_t P, uint32_t B) { return forward_moments(s, P, B); }
+int adjoint_mom(double s, uint64_t P, uint32_t B) { return adjoint_moments(s, P, B); }
+}
+"""
+
+
+def load():
+    d = tempfile.mkdtemp()
+    src, so = os.path.join(d, "rules.cpp"), os.path.join(d, "rules.so")
+    with open(src, "w") as f:
+        f.write(SRC)
+    inc = os.path.join(ROOT, "paper_2506_03747_gb300", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + inc, src, "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    lib.rows_per_bin.argtypes = lib.fits.argtypes = [ctypes.c_double]
+    lib.forward_mom.argtypes = lib.adjoint_mom.argtypes = [ctypes.c_double, ctypes.c_uint64, ctypes.c_uint32]
+    return lib
