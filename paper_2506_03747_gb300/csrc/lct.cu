@@ -173,10 +173,17 @@ __global__ void time_kernel(const double2* vol, LctDims d, float* tau) {
 // Bound: the FP64 pipe's N^4 additions (1.68 lanes a cycle and SM: 0.53 ms at
 // N = 128), taken about 1.3 times because a pixel's additions from one patch
 // can straddle two windows, and the warps in flight (shared memory holds 12
-// to 24). N = 128, M = 1024: 1.16 ms against 65.7 ms of the FFT form; N = 64:
-// 0.27 against 15.4; N = 16: 0.045 against 0.92. Patches of 32 x 1 columns and
-// 1 x 32 segments of pixels took 1.7 ms. Sums as two FP32 words would take
-// 0.73 ms at the same measured error, but carry 48 bits instead of 53.
+// to 24). N = 128, M = 1024: 1.2 to 1.4 ms over several runs against 65.7 ms of the
+// FFT form; N = 64: 0.29 against 15.4; N = 16: 0.04 against 0.92. Patches of 32 x 1
+// columns and 1 x 32 segments of pixels took 1.7 ms. Sums as two FP32 words would
+// take 0.73 ms at the same measured error, but carry 48 bits instead of 53.
+// On a rough map (silhouettes, noise) a block spans many windows, and visiting
+// all of its pixels in each costs 0.47 ms a window at N = 128, where one window's
+// additions cost 1.3. Blocks of more than 2.5 windows' rows have their pixels
+// tested one a lane first (0.05 ms a window, but 2.2 ms for additions that come
+// four at a time): uniformly random depths, N = 128, M = 1024: 3.0 ms against 8.3
+// with whole blocks; N = 512, M = 512: 477 against 1037 (FFTs 579); below 2.5 windows
+// whole blocks are faster (N = 128, M = 128: 1.65 against 2.29).
 // ---------------------------------------------------------------------------
 constexpr int kDirSide = 4;      // side of a block of pixels
 constexpr int kDirBins = 8;      // windows start at multiples of 8 bins (32-byte stores)
@@ -206,6 +213,7 @@ struct DirArgs {
   const DirWindow* win;
   float* tau;
   uint32_t N, M, n_seg, per_row;  // blocks of pixels; per_row along y
+  int wide;                // rows beyond which a block's pixels are tested one by one
   uint32_t py, px, n_py;   // patch of py columns along y and px along x; patches along y
 };
 
@@ -269,21 +277,30 @@ __global__ void __launch_bounds__(32) direct_kernel(const DirArgs a) {
   for (int i = 0; i < w.rows; ++i) hist[i * 32 + lane] = 0.0;
   const int16_t* at = a.node + (x + N) * n2 + y + N;
   double* h = hist + lane;
+  // the pixels [xa, xa + side) x [ya, ya + side) with rows [lo, hi]: can they reach
+  // the window from the patch? The node's offset grows with the distance from the
+  // centre; one row of slack on each side against its rounding.
+  auto reaches = [&](int xa, int ya, int side, int lo, int hi) {
+    const int dx0 = x0 - (xa + side - 1), dx1 = x1 - xa, dy0 = y0 - (ya + side - 1), dy1 = y1 - ya;
+    const int kn = a.node[(near_offset(dx0, dx1) + N) * n2 + near_offset(dy0, dy1) + N];
+    const int kf = a.node[(far_offset(dx0, dx1) + N) * n2 + far_offset(dy0, dy1) + N];
+    return kn != kNoNode && lo + kn - 1 < w.row0 + w.rows && hi + kf + 1 >= w.row0;
+  };
+  auto add = [&](const double2& q, int t) {
+    // no node: at least 0x7fff - 4096 rows beyond any window
+    const int r = __double2loint(q.y) + t - w.row0;
+    if ((unsigned)r < (unsigned)w.rows) h[r * 32] += q.x;
+  };
   for (uint32_t s0 = 0; s0 < a.n_seg; s0 += 32) {
     const uint32_t s = s0 + lane;
-    bool live = false;
+    bool live = false, wide = false;
     if (s < a.n_seg) {
       const int2 r = a.seg[s];
-      const int xs = (int)(s / a.per_row) * SIDE, ys = (int)(s % a.per_row) * SIDE;
-      const int xa = x0 - (xs + SIDE - 1), xb = x1 - xs, ya = y0 - (ys + SIDE - 1), yb = y1 - ys;
-      // the node's offset grows with the distance from the centre; one row of
-      // slack on each side against its rounding
-      const int kn = a.node[(near_offset(xa, xb) + N) * n2 + near_offset(ya, yb) + N];
-      const int kf = a.node[(far_offset(xa, xb) + N) * n2 + far_offset(ya, yb) + N];
-      live = r.x <= r.y && kn != kNoNode && r.x + kn - 1 < w.row0 + w.rows &&
-             r.y + kf + 1 >= w.row0;
+      live = r.x <= r.y && reaches((int)(s / a.per_row) * SIDE, (int)(s % a.per_row) * SIDE, SIDE,
+                                   r.x, r.y);
+      wide = SIDE == kDirSide && r.y - r.x > a.wide;
     }
-    for (uint32_t m = __ballot_sync(0xffffffffu, live); m; m &= m - 1) {
+    for (uint32_t m = __ballot_sync(0xffffffffu, live && !wide); m; m &= m - 1) {
       const uint32_t sl = s0 + __ffs(m) - 1;
       const int xs = (int)(sl / a.per_row) * SIDE, ys = (int)(sl % a.per_row) * SIDE;
       const double2* vp = reinterpret_cast<const double2*>(a.vox + sl * (SIDE * SIDE));
@@ -296,10 +313,40 @@ __global__ void __launch_bounds__(32) direct_kernel(const DirArgs a) {
         t[i] = (int)__ldg(kp - (i / SIDE) * n2 - i % SIDE);
       }
 #pragma unroll
-      for (int i = 0; i < SIDE * SIDE; ++i) {
-        // no node: at least 0x7fff - 4096 rows beyond any window
-        const int r = __double2loint(q[i].y) + t[i] - w.row0;
-        if ((unsigned)r < (unsigned)w.rows) h[r * 32] += q[i].x;
+      for (int i = 0; i < SIDE * SIDE; ++i) add(q[i], t[i]);
+    }
+    // two wide blocks at a time: each lane tests one pixel, and those that reach
+    // the window are taken four at a time
+    for (uint32_t m = __ballot_sync(0xffffffffu, live && wide); m;) {
+      const uint32_t sa = s0 + __ffs(m) - 1;
+      m &= m - 1;
+      const uint32_t sb = m ? s0 + __ffs(m) - 1 : sa;
+      const bool two = m != 0u;
+      m &= m - 1;
+      const uint32_t sl = lane < 16 ? sa : sb;
+      const int xp = (int)(sl / a.per_row) * SIDE + lane % 16 / SIDE;
+      const int yp = (int)(sl % a.per_row) * SIDE + lane % 16 % SIDE;
+      const int row = a.vox[sl * 16 + lane % 16].row;
+      const bool pix = (lane < 16 || two) && row != kNoRow && reaches(xp, yp, 1, row, row);
+      for (uint32_t mp = __ballot_sync(0xffffffffu, pix); mp;) {
+        double2 q[4];
+        int t[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          // (past the last one: a pixel without a surface)
+          q[i] = make_double2(0.0, __hiloint2double(0, kNoRow));
+          t[i] = 0;
+          if (mp) {
+            const uint32_t j = __ffs(mp) - 1, sj = j < 16 ? sa : sb, p = j % 16;
+            const int xj = (int)(sj / a.per_row) * SIDE + (int)p / SIDE;
+            const int yj = (int)(sj % a.per_row) * SIDE + (int)p % SIDE;
+            q[i] = __ldg(reinterpret_cast<const double2*>(a.vox + sj * 16 + p));
+            t[i] = (int)__ldg(at - (xj * n2 + yj));
+          }
+          mp &= mp - 1;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) add(q[i], t[i]);
       }
     }
   }
@@ -341,10 +388,12 @@ std::vector<DirWindow> dir_windows(int M, int max_rows) {
   return out;
 }
 
-// The direct form's N^4 additions (4.3 ps each) against the FFT form's passes
-// over 8 N^2 M padded samples (about 490 ps each): direct below N^2 of about
-// 900 M. Measured on both sides of the line: N = 128, M = 64: 1.16 against 3.9
-// ms, M = 16: 1.2 against 1.39; N = 256, M = 64: 18 against 16.
+// The direct form's N^4 additions (4.3 ps each on a smooth map) against the FFT
+// form's passes over 8 N^2 M padded samples (about 490 ps each): direct below N^2 of
+// about 900 M. Measured on both sides of the line: N = 128, M = 64: 1.16 against 3.9
+// ms, M = 16: 1.2 against 1.39; N = 256, M = 64: 18 against 16. On random depths the
+// direct form is also the faster one up to the line: N = 128, M = 32: 1.34 against
+// 2.04 ms; N = 256, M = 128: 25 against 32; N = 512, M = 512: 477 against 579.
 bool direct_form(uint32_t N, uint32_t M) { return (uint64_t)N * N <= 900ull * M; }
 
 bool pow2(uint32_t v) { return v >= 2 && (v & (v - 1)) == 0; }
@@ -444,6 +493,7 @@ cudaError_t create_direct(nlos_lct* p, double slope4sq, cudaStream_t st) {
   a.py = std::min(d.N, 8u);
   a.px = 32u / a.py;
   a.n_py = d.N / a.py;
+  a.wide = dir_rows(d.N) * 5 / 2;
   const std::vector<DirWindow> win = dir_windows((int)d.M, dir_rows(d.N));
   std::vector<double> weight(d.M);
   for (uint32_t z = 0; z < d.M; ++z) {
