@@ -105,8 +105,8 @@ struct SceneScratch {
   unsigned long long boundary_pairs;
   unsigned long long pairs_full;  // pairs through the full evaluation (past the early out)
   unsigned long long next_chunk;  // forward: next chunk of work units to claim
-  unsigned long long pairs_tested;  // pairs of the units the forward staged
-  unsigned long long n_live;      // forward: entries of its live-unit list
+  unsigned long long pairs_tested;  // pairs of the groups the forward staged
+  unsigned long long n_live;      // forward: its live-unit list's entries (low word) and weight (high)
   // --- reset by the detector as well from here: its results ---
   unsigned int peak_bits;     // max of tau_G as float bits (values are >= 0)
   unsigned int pad2;

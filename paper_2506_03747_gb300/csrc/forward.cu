@@ -476,12 +476,7 @@ cudaError_t forward_plan_create(SceneImpl& sc) {
     a.n_win = (g.B + max_bw - 1) / max_bw;
     a.bw = ((g.B + a.n_win - 1) / a.n_win + 3) & ~3u;
   }
-  // a scene of few units is cut into smaller blocks, so that more SMs take part
-  // (the 32 x 32 scan of 1,024 points has 32 units of 1,024: 32.1 us a pass in one
-  // block, 22 us in blocks of 128 points)
-  while (a.ppb > kFwdMinPpb && n_tiles * a.n_win * ((a.n_pairs + a.ppb - 1) / a.ppb) <
-                                   (uint64_t)sc.num_sms)
-    a.ppb /= 2;
+  a.ppb = block_pairs(a.ppb, n_tiles, a.n_win, a.n_pairs, (uint64_t)sc.num_sms);
   p->smem = (moments ? (size_t)kMoments * kMomRows : (size_t)a.bw) * kTile * 4 + stage_bytes();
   a.n_blk = (a.n_pairs + a.ppb - 1) / a.ppb;
   a.units = (unsigned long long)n_tiles * a.n_win * a.n_blk;

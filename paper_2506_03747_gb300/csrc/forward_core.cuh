@@ -73,7 +73,6 @@ constexpr int kPairsPerBlock = 256;         // serving kernel: 16 KB per staged 
 #define NLOS_FWD_UNROLL 4                   // standalone forward: unroll of the pair loop
 #endif
 
-constexpr uint32_t kFwdMinPpb = 64;  // smallest block of a scene of few units
 constexpr int kFwdUnroll = NLOS_FWD_UNROLL;  // (#pragma unroll takes no macro)
 
 enum { MODE_NEAREST = 0, MODE_NEAREST_COUNT = 1, MODE_SPLAT = 2, MODE_SPLAT_MOM = 3,

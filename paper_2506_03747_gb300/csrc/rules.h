@@ -57,4 +57,16 @@ inline bool adjoint_moments(double sigma, uint64_t P, uint32_t B) {
   return P >= (B > kAdjOneCtaBins ? 1ull : 4ull) * (uint64_t)q * B;
 }
 
+// Pairs of a staged block: `most`, halved while the scene has fewer units (tile,
+// window, block) than SMs, so that more SMs take part (the 32 x 32 scan of 1,024
+// points has 32 units of 1,024: 32.1 us a pass in one block, 22 us in blocks of 128
+// points).
+constexpr uint32_t kFwdMinPpb = 64;
+inline uint32_t block_pairs(uint32_t most, uint64_t n_tiles, uint64_t n_win, uint64_t n_pairs,
+                            uint64_t sms) {
+  uint32_t ppb = most;
+  while (ppb > kFwdMinPpb && n_tiles * n_win * ((n_pairs + ppb - 1) / ppb) < sms) ppb /= 2;
+  return ppb;
+}
+
 }  // namespace nlos

@@ -14,6 +14,9 @@ int fits(double s) { return moments_fit(s); }
 int max_j() { return kMomMaxJ; }
 int max_taps() { return kMomTaps; }
 int forward_mom(double s, uint64_t P, uint32_t B) { return forward_moments(s, P, B); }
+uint32_t pairs_of_block(uint32_t most, uint32_t t, uint32_t w, uint32_t n, uint32_t sms) {
+  return block_pairs(most, t, w, n, sms);
+}
 int adjoint_mom(double s, uint64_t P, uint32_t B) { return adjoint_moments(s, P, B); }
 }
 """
