@@ -242,9 +242,12 @@ nlos_status nlos_scene_shape(const nlos_scene* scene, uint64_t* num_scan, uint32
  * Asynchronous on cuda_stream otherwise. Calls on one scene must not overlap
  * on the device (they share its scratch): use one stream per scene.
  * Device memory: the forward's live-unit list (16 bytes a (tile, window, point
- * block) unit) and the noise step's deferred-bin lists (about 3% of the bins;
- * noise_mode != NONE) belong to the scene from its creation, whose calls
- * allocate nothing. */
+ * block) unit, at most 64 MiB, in passes beyond) and the noise step's
+ * deferred-bin lists (about 3% of the bins; noise_mode != NONE) belong to the
+ * scene from its creation, and its calls allocate nothing. Where there was no
+ * memory for them, the scene works without: the forward tests the units itself,
+ * and the noise step takes its lists from the stream's pool (cudaMallocAsync) or
+ * samples in one pass. */
 nlos_status nlos_simulate(nlos_scene* scene, float* tau_dev, uint32_t* counts_dev,
                           double* energy_dev, nlos_stats* stats, void* cuda_stream);
 

@@ -104,8 +104,9 @@ struct SceneScratch {
   // --- reset per forward pass from here: its counters ---
   unsigned long long boundary_pairs;
   unsigned long long pairs_full;  // pairs through the full evaluation (past the early out)
-  unsigned long long next_chunk;  // forward: next chunk of work units to claim
   unsigned long long pairs_tested;  // pairs of the groups the forward staged
+  // (next_chunk and n_live: zeroed for each pass over the list)
+  unsigned long long next_chunk;  // forward: next chunk of work units to claim
   unsigned long long n_live;      // forward: its live-unit list's entries (low word) and weight (high)
   // --- reset by the detector as well from here: its results ---
   unsigned int peak_bits;     // max of tau_G as float bits (values are >= 0)

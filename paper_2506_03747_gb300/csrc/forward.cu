@@ -79,7 +79,8 @@ constexpr int kListThreads = 1024;  // (of fewer blocks than 128 a tile: 256)
 // (tile, window) are contiguous (a CTA's blocks at a time), so a range of the list
 // rarely spans many tiles; the order of the runs does not matter. Each entry
 // holds the weight of the list before it (both come from one atomic, so they
-// ascend together). The same launch zeroes the output that the forward adds to.
+// ascend together). The same launch zeroes the output that the forward adds to
+// (of a list in several passes, a memory set does).
 template <int SCAN, int COS, int MODE>
 __global__ void __launch_bounds__(kListThreads)
     unit_list_kernel(const __grid_constant__ FwdArgs a, ListEntry* __restrict__ list,
@@ -87,9 +88,11 @@ __global__ void __launch_bounds__(kListThreads)
   __shared__ uint32_t s_units[32], s_groups[32], s_n;
   __shared__ uint32_t s_blk[kListThreads], s_rows[kListThreads], s_mask[kListThreads];
   __shared__ unsigned long long s_base;
-  zero_floats(a.tau, (size_t)a.S * a.B);
-  if (MODE == MODE_SPLAT_MOM) zero_floats(a.far_mass, a.S);
-  const unsigned long long tw = blockIdx.x;
+  if (a.list_zeroes) {
+    zero_floats(a.tau, (size_t)a.S * a.B);
+    if (MODE == MODE_SPLAT_MOM) zero_floats(a.far_mass, a.S);
+  }
+  const unsigned long long tw = a.list_tw0 + blockIdx.x;
   const float margin = window_margin<MODE>(a);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const TileBound tile = a.tiles[(uint32_t)(tw / a.n_win)];
@@ -348,7 +351,8 @@ struct FwdPlan {
   ListFn list_fn = nullptr;  // null: chunks of all units are claimed
   size_t smem = 0;
   unsigned grid = 0;
-  ListEntry* list = nullptr;  // [units], or null
+  ListEntry* list = nullptr;  // [pass_runs * n_blk], or null
+  uint64_t pass_runs = 0;     // (tile, window) runs of a pass over the list
 };
 
 namespace {
@@ -493,9 +497,10 @@ cudaError_t forward_plan_create(SceneImpl& sc) {
   // units of which most may be culled, so tile changes (flush, zeroing,
   // barriers) are fewer per unit of work. Without memory for it the producers
   // test the units themselves.
+  p->pass_runs = list_pass_runs(a.units / a.n_blk, a.n_blk);
   if (NLOS_FWD_CULL && mode != MODE_NEAREST_COUNT && a.units < (1ull << 32) &&
-      cudaMalloc(reinterpret_cast<void**>(&p->list), sizeof(ListEntry) * a.units) !=
-          cudaSuccess) {
+      cudaMalloc(reinterpret_cast<void**>(&p->list),
+                 sizeof(ListEntry) * p->pass_runs * a.n_blk) != cudaSuccess) {
     p->list = nullptr;
     (void)cudaGetLastError();
   }
@@ -520,20 +525,32 @@ cudaError_t launch_forward(const SceneImpl& sc, float* tau, cudaStream_t st) {
   if (p && p->mode != forward_mode(sc) &&
       (e = plan_mode(*p, sc, forward_mode(sc))) != cudaSuccess)
     return e;
-  if (!p || !p->list_fn) e = cudaMemsetAsync(tau, 0, sizeof(float) * g.S * g.B, st);
-  if (p && !p->list_fn && p->a.far_mass && e == cudaSuccess)
+  const uint64_t runs = p ? p->a.units / p->a.n_blk : 0;
+  const bool listed = p && p->list_fn;
+  const bool one_pass = listed && p->pass_runs == runs;  // whose list kernel zeroes the output
+  if (e == cudaSuccess && !one_pass) e = cudaMemsetAsync(tau, 0, sizeof(float) * g.S * g.B, st);
+  if (e == cudaSuccess && !one_pass && p && p->a.far_mass)
     e = cudaMemsetAsync(p->a.far_mass, 0, sizeof(float) * g.S, st);
   if (e != cudaSuccess || !p) return e;
   FwdArgs a = p->a;
   a.tau = tau;
-  if (p->list_fn) {
-    // (the counters, n_live among them, were zeroed with the pass's scratch)
-    p->list_fn<<<(unsigned)(a.units / a.n_blk), a.n_blk < 128 ? 256 : kListThreads, 0, st>>>(
-        a, p->list, &sc.scratch->n_live);
+  a.list_zeroes = one_pass ? 1u : 0u;
+  static_assert(offsetof(SceneScratch, n_live) == offsetof(SceneScratch, next_chunk) + 8,
+                "zeroed together");
+  // (the first pass finds its counters zeroed with the call's scratch)
+  for (uint64_t r = 0; r < (listed ? runs : 1); r += p->pass_runs) {
+    if (listed) {
+      a.list_tw0 = r;
+      if (r > 0 && (e = cudaMemsetAsync(a.next_chunk, 0, 2 * sizeof(unsigned long long), st)) !=
+                       cudaSuccess)
+        return e;
+      p->list_fn<<<(unsigned)std::min(p->pass_runs, runs - r), a.n_blk < 128 ? 256 : kListThreads,
+                   0, st>>>(a, p->list, &sc.scratch->n_live);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    p->fn<<<p->grid, 1024, p->smem, st>>>(a, p->mt, sc.occ);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  p->fn<<<p->grid, 1024, p->smem, st>>>(a, p->mt, sc.occ);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (p->mode == MODE_SPLAT_MOM) {
     const unsigned blocks = (unsigned)std::min<uint64_t>((g.S + 7) / 8, (uint64_t)sc.num_sms * 8);
     pick_tail(g.scan_mode, g.cos_mode)<<<blocks, 256, 0, st>>>(a);

@@ -145,6 +145,8 @@ struct FwdArgs {
   const ListEntry* unit_list;
   const unsigned long long* n_live;
   uint32_t list_shift;
+  unsigned long long list_tw0;   // first (tile, window) of the list's pass
+  uint32_t list_zeroes;          // the list's kernel zeroes the output (one pass only)
   uint32_t list_chunks_per_cta;  // list chunks per CTA (mean), of the claimed part
   uint32_t list_min_chunk, list_max_chunk;  // list entries per chunk, clamped
   uint32_t list_static_pct;  // the list's first part (percent of weight) in one range per CTA

@@ -17,6 +17,8 @@ int forward_mom(double s, uint64_t P, uint32_t B) { return forward_moments(s, P,
 uint32_t pairs_of_block(uint32_t most, uint32_t t, uint32_t w, uint32_t n, uint32_t sms) {
   return block_pairs(most, t, w, n, sms);
 }
+uint64_t pass_runs(uint64_t runs, uint64_t n_blk) { return list_pass_runs(runs, n_blk); }
+uint64_t list_entries() { return kListEntries; }
 int adjoint_mom(double s, uint64_t P, uint32_t B) { return adjoint_moments(s, P, B); }
 }
 """
@@ -32,4 +34,6 @@ def load():
     lib = ctypes.CDLL(so)
     lib.rows_per_bin.argtypes = lib.fits.argtypes = [ctypes.c_double]
     lib.forward_mom.argtypes = lib.adjoint_mom.argtypes = [ctypes.c_double, ctypes.c_uint64, ctypes.c_uint32]
+    lib.pass_runs.argtypes = [ctypes.c_uint64, ctypes.c_uint64]
+    lib.pass_runs.restype = lib.list_entries.restype = ctypes.c_uint64
     return lib

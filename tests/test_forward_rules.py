@@ -1,5 +1,6 @@
 """The forward's sizing rules (host, no GPU): blocks shrink for scenes of few
-units only, also where the number of units passes 2^32."""
+units only, also where the number of units passes 2^32; the live-unit list is
+bounded and its passes cover every run."""
 import pytest
 
 from tests import rules_lib
@@ -24,3 +25,15 @@ def test_small_blocks_for_few_units(rules):
 def test_many_units_keep_whole_blocks(rules, tiles, windows, pairs):
     assert (tiles * windows * -(-pairs // 512)) % (1 << 32) < 152 or pairs == (1 << 30) - 1
     assert rules.pairs_of_block(512, tiles, windows, pairs, 152) == 512
+
+
+@pytest.mark.parametrize("runs,blocks", [(1, 1), (512, 1024), (4096, 1024), (4097, 1024), (2048, 16384),
+                                         (7, 1 << 22), (7, (1 << 22) + 1), (3, 1 << 23), (17477, 240),
+                                         ((1 << 32) - 1, 1)])
+def test_list_passes(rules, runs, blocks):
+    per = rules.pass_runs(runs, blocks)
+    most = max(1, rules.list_entries() // blocks)
+    assert 1 <= per <= most
+    passes = -(-runs // per)
+    assert passes == -(-runs // most)  # no more of them than the bound asks for
+    assert runs * blocks > rules.list_entries() or passes == 1
