@@ -21,10 +21,16 @@
 //     ordering.
 // The steps are short whatever the point count, so what they cost is launches
 // and latency: as six kernels 45 us for 262,144 points and 32 us for 40,001.
+// The barriers need every CTA resident, which a cooperative launch promises on
+// the context's SMs. On a stream of a green context, which may have only some of
+// them, and where the launch is refused, the same four steps are four launches of
+// their own.
 #include "common.cuh"
 #include "order_core.cuh"
 #include "device_util.cuh"
 #include "pack_core.cuh"
+
+#include <cuda.h>
 
 #include <algorithm>
 #include <cmath>
@@ -64,10 +70,13 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* word, unsigned int* err) 
 
 constexpr int kOrderThreads = 512;
 
+// GRID: all steps with grid barriers between them (a cooperative launch); else
+// the one step `step`.
+template <bool GRID>
 __global__ void __launch_bounds__(kOrderThreads, 2)
     order_kernel(const float* __restrict__ raw, uint64_t P, int scan_mode, int cos_mode,
                  const PackConst pc, uint16_t* cell, uint32_t* counts, uint32_t* perm,
-                 unsigned int* err) {
+                 unsigned int* err, int step) {
   __shared__ uint32_t red[kOrderThreads / 32 * 6];
   __shared__ uint32_t base[kOrderCells / kSliceCells];
   uint32_t* box = counts + kOrderCells;
@@ -75,12 +84,14 @@ __global__ void __launch_bounds__(kOrderThreads, 2)
   const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  box_range(raw, 0, P, t, stride, box, red);
-  if (!grid_barrier(box + kBarrierWord, err)) return;
-  cell_range(raw, 0, P, t, stride, box, cell, counts, scan_mode, cos_mode, pc);
-  if (!grid_barrier(box + kBarrierWord, err)) return;
+  if (GRID || step == 0) box_range(raw, 0, P, t, stride, box, red);
+  if (GRID && !grid_barrier(box + kBarrierWord, err)) return;
+  if (GRID || step == 1)
+    cell_range(raw, 0, P, t, stride, box, cell, counts, scan_mode, cos_mode, pc);
+  if (GRID && !grid_barrier(box + kBarrierWord, err)) return;
   // a warp scans 64 cells of a slice, then the 16 warp totals are scanned
-  for (uint32_t sl = blockIdx.x; sl < kOrderCells / kSliceCells; sl += gridDim.x) {
+  for (uint32_t sl = GRID || step == 2 ? blockIdx.x : kOrderCells;
+       sl < kOrderCells / kSliceCells; sl += gridDim.x) {
     uint32_t* seg = counts + sl * kSliceCells + w * 64;
     const uint32_t v0 = seg[lane], v1 = seg[32 + lane];
     const uint32_t x0 = inclusive_scan(v0);
@@ -98,7 +109,8 @@ __global__ void __launch_bounds__(kOrderThreads, 2)
     seg[32 + lane] = red[w] + x1 - v1;
     __syncthreads();
   }
-  if (!grid_barrier(box + kBarrierWord, err)) return;
+  if (GRID && !grid_barrier(box + kBarrierWord, err)) return;
+  if (!GRID && step != 3) return;
   if (w == 0) {
     const uint32_t v = *(volatile uint32_t*)&totals[lane];
     base[lane] = inclusive_scan(v) - v;
@@ -176,6 +188,24 @@ __global__ void __launch_bounds__(kSubPairs) pack_bounds_kernel(
   }
 }
 
+// Whether a stream belongs to a green context (or the driver does not say).
+bool partitioned(cudaStream_t st) {
+  using StreamGetCtx = decltype(&cuStreamGetCtx_v2);
+  static const StreamGetCtx stream_ctx = [] {
+    void* q = nullptr;
+    cudaDriverEntryPointQueryResult r = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuStreamGetCtx", &q, 13000, cudaEnableDefault, &r) ==
+            cudaSuccess &&
+        r == cudaDriverEntryPointSuccess)
+      return reinterpret_cast<StreamGetCtx>(q);
+    (void)cudaGetLastError();
+    return StreamGetCtx(nullptr);
+  }();
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  return !stream_ctx || stream_ctx(st, &ctx, &green) != CUDA_SUCCESS || green;
+}
+
 }  // namespace
 
 cudaError_t init_order(SceneImpl& s, cudaStream_t st) {
@@ -194,17 +224,29 @@ cudaError_t launch_order_pack(SceneImpl& s, cudaStream_t st) {
   if (P == 0) return cudaSuccess;
   uint32_t* counts = s.cells;
   const PackConst pc = pack_const(s.params.laser_x, s.params.laser_y, 1.0 / g.cdt);
-  // one wave (the barriers need every CTA resident), at least a CTA a slice
-  unsigned grid = (unsigned)std::min<uint64_t>(
-      std::max<uint64_t>((P + kOrderThreads - 1) / kOrderThreads, kOrderCells / kSliceCells),
-      (uint64_t)s.num_sms * 2);
-  uint64_t n = P;
-  int scan_mode = g.scan_mode, cos_mode = g.cos_mode;
+  // one wave, at least a CTA a slice
+  const uint64_t want =
+      std::max<uint64_t>((P + kOrderThreads - 1) / kOrderThreads, kOrderCells / kSliceCells);
+  const unsigned grid = (unsigned)std::min<uint64_t>(want, 2ull * (unsigned)s.num_sms);
   unsigned int* err = &s.scratch->err;
-  void* args[] = {&s.raw_points, &n, &scan_mode, &cos_mode, const_cast<PackConst*>(&pc),
-                  &s.cell, &counts, &s.perm, &err};
-  cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&order_kernel), dim3(grid),
-                                              dim3(kOrderThreads), args, 0, st);
+  cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+  if (!partitioned(st)) {
+    uint64_t n = P;
+    int scan_mode = g.scan_mode, cos_mode = g.cos_mode, step = 0;
+    void* args[] = {&s.raw_points, &n, &scan_mode, &cos_mode, const_cast<PackConst*>(&pc),
+                    &s.cell, &counts, &s.perm, &err, &step};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&order_kernel<true>), dim3(grid),
+                                    dim3(kOrderThreads), args, 0, st);
+  }
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    (void)cudaGetLastError();
+    e = cudaSuccess;
+    for (int step = 0; step < 4 && e == cudaSuccess; ++step) {
+      order_kernel<false><<<grid, kOrderThreads, 0, st>>>(s.raw_points, P, g.scan_mode, g.cos_mode,
+                                                          pc, s.cell, counts, s.perm, err, step);
+      e = cudaGetLastError();
+    }
+  }
   if (e != cudaSuccess) return e;
   const uint64_t n_pairs = (P + 1) / 2;
   const uint64_t n_sub = (n_pairs + kSubPairs - 1) / kSubPairs;
