@@ -74,7 +74,10 @@ using JitterLong = JitterArgs<kJitterMaxTaps>;
 //    threads' overlap hits L1), so no barrier separates loads and stores;
 //  * other rows (bin counts that are not multiples of 4, unaligned buffers)
 //    and radii above 16: a run of the trace with its halo is staged in shared
-//    memory by coalesced loads, and each thread takes 4 bins from it.
+//    memory by coalesced loads, and each thread takes 4 bins from it. Above 16 the
+//    loop over the taps reads the halo as 16-byte words (16,384 x 1024 bins, R = 40:
+//    106 us, R = 200: 381 us; with one word a tap 160 and 701, and one bin a
+//    thread 157 and 698). Bound: FMA issue and the taps' indexed constant loads.
 // Every bin adds its taps in the same order in all forms.
 template <int R>
 __global__ void __launch_bounds__(256) jitter_direct_kernel(const __grid_constant__ JitterShort a) {
@@ -146,20 +149,32 @@ __global__ void __launch_bounds__(256) jitter_kernel(const __grid_constant__ Arg
 #pragma unroll
       for (int j = -RT; j <= RT; ++j) acc[e] = fmaf(a.taps[j + RT], x[4 * kQ + e - j], acc[e]);
   } else {
-    // out[b] = sum_j taps[j + R] * in[b - j]; in[b - j] sits at sm[o + e + halo - j]
+    // out[b] = sum_j taps[j + R] * in[b - j]; in[b - j] sits at sm[o + e + halo - j].
+    // Four taps take the seven inputs of two 16-byte words, one of them new (read
+    // one by one, a warp's inputs 16 bytes apart met in the same banks).
     const float* c = sm + o + halo;
-    float x0 = c[R], x1 = c[R + 1], x2 = c[R + 2], x3 = c[R + 3];
-    for (int j = -R; j <= R; ++j) {
+    int j = -R;
+    auto one = [&]() {
       const float g = a.taps[j + R];
-      acc[0] = fmaf(g, x0, acc[0]);
-      acc[1] = fmaf(g, x1, acc[1]);
-      acc[2] = fmaf(g, x2, acc[2]);
-      acc[3] = fmaf(g, x3, acc[3]);
-      x3 = x2;
-      x2 = x1;
-      x1 = x0;
-      x0 = j < R ? c[-j - 1] : 0.0f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[e] = fmaf(g, c[e - j], acc[e]);
+      ++j;
+    };
+    while (j & 3) one();
+    float4 hi = *reinterpret_cast<const float4*>(c - j);
+#pragma unroll 4
+    for (; j + 3 <= R; j += 4) {
+      const float4 lo = *reinterpret_cast<const float4*>(c - j - 4);
+      const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float g = a.taps[j + k + R];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[e] = fmaf(g, x[4 + e - k], acc[e]);
+      }
+      hi = lo;
     }
+    while (j <= R) one();
   }
   float* orow = a.out + t * a.B + b0;
 #pragma unroll
