@@ -146,7 +146,7 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-FORWARD_SOURCES = ("forward.cu", "forward_core.cuh", "device_util.cuh", "common.cuh")
+FORWARD_SOURCES = ("forward.cu", "forward_core.cuh", "rules.h", "device_util.cuh", "common.cuh")
 # FP32 issue slots of the moment-form adjoint: of every (scan point, point) pair
 # (differences 2, squared length 3, reciprocal square root step and length 4,
 # path bin 1), and of a pair that reaches the window and faces its spot

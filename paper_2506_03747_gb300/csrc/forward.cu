@@ -7,16 +7,18 @@
 //  * One CTA tile = 32 scan points; lane l of every warp owns scan point l of
 //    the tile, so the shared histogram [bin][32] gives every lane its own bank
 //    and the shared atomics of a warp never conflict.
-//  * Surface points are packed in pairs (64 B, see PointPair) and staged into
-//    shared memory by 1-D TMA bulk copies, double-buffered on mbarriers. All
-//    warps of the CTA read the same staged block (broadcast loads) and split
-//    its pairs; each lane evaluates the two points of a pair for its scan
-//    point with packed FP32x2 arithmetic (__ffma2_rn & co.).
-//  * Work units (scan tile, bin window, point block) are split evenly over a
-//    persistent grid (stream-K): a CTA flushes its partial histogram into the
-//    zeroed output with vectorised global reductions whenever its (tile,
-//    window) changes. The jitter convolution is linear, so it is applied to
-//    each partial histogram during the flush.
+//  * Surface points are packed in pairs (64 B, see PointPair). One producer warp
+//    stages the groups of 16 pairs that the tile may bin into shared memory by
+//    1-D TMA bulk copies, a few slots ahead on mbarriers; the other warps read the
+//    same slot (broadcast loads) and split its pairs; each lane evaluates the two
+//    points of a pair for its scan point with packed FP32x2 arithmetic
+//    (__ffma2_rn & co.).
+//  * Work units (scan tile, bin window, point block): a first kernel lists those
+//    that the bounds leave, and a persistent grid takes the list in contiguous
+//    ranges of equal weight, the rest of a long list in claimed chunks. A CTA
+//    flushes its partial histogram into the zeroed output with vectorised global
+//    reductions whenever its (tile, window) changes. The jitter convolution is
+//    linear, so it is applied to each partial histogram during the flush.
 #include "forward_core.cuh"
 #include "pack_core.cuh"
 
@@ -24,8 +26,9 @@
 
 namespace nlos {
 
-// Standalone launch: a persistent grid (one CTA per SM) claims chunks of the
-// job's work units from a counter in the scene scratch.
+// Standalone launch: a persistent grid (one CTA per SM) over the live-unit list
+// or, without one, over chunks of all units claimed from a counter in the scene
+// scratch.
 template <int SCAN, int COS, int MODE>
 __global__ void __launch_bounds__(1024, 1)
     fwd_kernel(const __grid_constant__ FwdArgs a, const __grid_constant__ MomTab mt,

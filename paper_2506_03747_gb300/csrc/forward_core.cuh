@@ -10,15 +10,14 @@
 //    tile, so the shared histogram [bin][32] gives every lane its own bank and
 //    the shared atomics of a warp never conflict.
 //  * Surface points are packed in pairs (64 B, PointPair) and staged into
-//    shared memory by 1-D TMA bulk copies, double-buffered on mbarriers. All
-//    warps of the CTA read the same staged block (broadcast loads) and split
+//    shared memory by 1-D TMA bulk copies, into a few slots on mbarriers. All
+//    consumer warps of the CTA read the same slot (broadcast loads) and split
 //    its pairs; each lane evaluates the two points of a pair for its scan
 //    point with packed FP32x2 arithmetic (__ffma2_rn & co.).
-//  * A work unit is (scan tile, bin window, point block). A CTA runs a
-//    contiguous range of units and flushes its partial histogram into the
-//    zeroed output with vectorised global reductions whenever its (tile,
-//    window) changes; the jitter convolution is linear, so it is applied to
-//    each partial histogram during the flush.
+//  * A work unit is (scan tile, bin window, point block). A CTA flushes its
+//    partial histogram into the zeroed output with vectorised global reductions
+//    whenever its (tile, window) changes; the jitter convolution is linear, so
+//    it is applied to each partial histogram during the flush.
 #pragma once
 
 #include "common.cuh"
