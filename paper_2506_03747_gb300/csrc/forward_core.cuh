@@ -144,8 +144,6 @@ struct FwdArgs {
   const ListEntry* unit_list;
   const unsigned long long* n_live;
   uint32_t list_shift;
-  unsigned long long list_tw0;   // first (tile, window) of the list's pass
-  uint32_t list_zeroes;          // the list's kernel zeroes the output (one pass only)
   uint32_t list_chunks_per_cta;  // list chunks per CTA (mean), of the claimed part
   uint32_t list_min_chunk, list_max_chunk;  // list entries per chunk, clamped
   uint32_t list_static_pct;  // the list's first part (percent of weight) in one range per CTA
@@ -163,6 +161,10 @@ struct FwdArgs {
   float taps[kMaxTaps];
   int replicate;     // jitter with the edge bins continued outside the window
   float tail[kMaxTaps / 2 + 1];  // replicate corrections (jitter_tails)
+  // the list's kernel: first (tile, window) of the pass, and whether it zeroes the
+  // output (of a list in one pass)
+  unsigned long long list_tw0;
+  uint32_t list_zeroes;
 };
 
 struct bool2_t {
