@@ -390,10 +390,10 @@ std::vector<DirWindow> dir_windows(int M, int max_rows) {
 
 // The direct form's N^4 additions (4.3 ps each on a smooth map) against the FFT
 // form's passes over 8 N^2 M padded samples (about 490 ps each): direct below N^2 of
-// about 900 M. Measured on both sides of the line: N = 128, M = 64: 1.16 against 3.9
-// ms, M = 16: 1.2 against 1.39; N = 256, M = 64: 18 against 16. On random depths the
-// direct form is also the faster one up to the line: N = 128, M = 32: 1.34 against
-// 2.04 ms; N = 256, M = 128: 25 against 32; N = 512, M = 512: 477 against 579.
+// about 900 M. Measured on both sides of the line, smooth maps: N = 128, M = 32: 1.34
+// against 2.04 ms, M = 16: 1.2 against 1.39; N = 256, M = 128: 14.6 against 32, M = 64:
+// 18 against 16. Random depths: N = 128, M = 32: 1.34 against 2.04 ms; N = 256, M = 128:
+// 25 against 32; N = 512, M = 512: 477 against 579.
 bool direct_form(uint32_t N, uint32_t M) { return (uint64_t)N * N <= 900ull * M; }
 
 bool pow2(uint32_t v) { return v >= 2 && (v & (v - 1)) == 0; }
